@@ -93,6 +93,27 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same wait by a converged warp: every lane polls, and the vote makes the
+// result warp-uniform, so a timeout never splits the warp.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, void* ws,
+                                               uint32_t site) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, ws, site));
+}
+
+// True in one lane of a converged warp (always the same lane).  The UMMA
+// issuers run as whole warps and issue under this predicate: the compiler then
+// knows that one thread executes the block and keeps descriptors in uniform
+// registers; under `lane == 0` it serialises every tcgen05.mma and commit.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ------------------------------------------------------------ CTA clusters
 // Rank of this CTA in its cluster, the shared::cluster address of the same
 // shared-memory offset in CTA `rank`, and the cluster-scope forms of the

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   __nv_bfloat16* __restrict__ dV) {
   using C = BCfg<D, PS, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (ws_failed(a.ws)) return;
   if (smem_u32(smem) & 1023u) {
     if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB11u);
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
         if (hc > 0) mbar_wait_bounded(q_full, uint32_t(hc - 1) & 1u, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ---------------------------------------------------------- UMMA issuer
       constexpr uint32_t idSP = idesc_bf16(128, PS, 0, 0);      // [tok x P], K = d
       constexpr uint32_t idTD = idesc_bf16(128, D, 0, 1);       // [tok x d], K = prototypes
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int hc = 0, gc = 0, hp = 0, gbuf = 0;
       bool ok = true;
       auto wt = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return ok = ok && mbar_wait(bar, par, abort_flag, a.ws, site);
+        return ok = ok && mbar_wait_warp(bar, par, abort_flag, a.ws, site);
       };
       auto sdcol = [&](int i) { return uint32_t(C::SD_COL + (i % C::NSD) * PS); };
       // operand descriptors built once and stepped by constant offsets: each
@@ -233,10 +233,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       wt(ring_full(0), 0, 0x502);
       if (ok) {
         tc_fence_after();
-        issue_S(0, sdcol(0));
-        umma_commit(s_full);
-        // slice mode: Q is read only by S, so it may be replaced after the last S of a head
-        if (MODE == kSlice && (ntiles == 1 || nxt.qk != cur.qk)) umma_commit(q_empty);
+        if (elect_one()) {
+          issue_S(0, sdcol(0));
+          umma_commit(s_full);
+          // slice mode: Q is read only by S, so it may be replaced after the last S of a head
+          if (MODE == kSlice && (ntiles == 1 || nxt.qk != cur.qk)) umma_commit(q_empty);
+        }
       }
       bool first_of_hp = true;
       for (int li = 0; li < ntiles && ok; ++li) {
@@ -253,30 +255,32 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) break;
         tc_fence_after();
         const uint32_t gofs = uint32_t(gbuf * C::Q_BYTES);  // this segment's dsketch buffer
-        {
+        if (elect_one()) {
           const uint64_t dVk = sdesc_add(dRk, uint32_t(sV) * C::KV_TILE), dG = sdesc_add(dGk, gofs);
 #pragma unroll
           for (int k = 0; k < D / 16; ++k)
             umma_ss(tmem + sdcol(li), sdesc_add(dVk, (k >> 2) * (T * 128) + (k & 3) * 32),
                     sdesc_add(dG, (k >> 2) * (PS * 128) + (k & 3) * 32), idSP, k > 0 ? 1u : 0u);
+          umma_commit(da_full);
+          if (MODE == kSlice) umma_commit(ring_empty(sV));
         }
-        umma_commit(da_full);
-        if (MODE == kSlice) umma_commit(ring_empty(sV));
         // ---- dV(i) = A G
         if (MODE == kFull) {
           wt(a_full, li & 1, 0x506);
           if (li > 0) wt(dv_empty, (li - 1) & 1, 0x507);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t dG = sdesc_add(dGm, gofs);
+          if (elect_one()) {
+            const uint64_t dG = sdesc_add(dGm, gofs);
 #pragma unroll
-          for (int k = 0; k < PS / 16; ++k)
-            umma_ss(tmem + C::DV_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dG, k * 2048),
-                    idTD, k > 0 ? 1u : 0u);
-          umma_commit(dv_full);
+            for (int k = 0; k < PS / 16; ++k)
+              umma_ss(tmem + C::DV_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dG, k * 2048),
+                      idTD, k > 0 ? 1u : 0u);
+            umma_commit(dv_full);
+          }
         }
         if (!ok) break;
-        if (cur.seg_last) umma_commit(g_empty_of(gbuf));
+        if (cur.seg_last && elect_one()) umma_commit(g_empty_of(gbuf));
         const bool more = li + 1 < ntiles;
         const bool newhead = more && nxt.qk != cur.qk;
         // ---- S(i+1) before dK/dQ(i) when its buffer and Q allow it
@@ -294,9 +298,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x50A);
           if (!ok) break;
           tc_fence_after();
-          issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
-          umma_commit(s_full);
-          if (MODE == kSlice && (li + 2 >= ntiles || nx2.qk != nxt.qk)) umma_commit(q_empty);
+          if (elect_one()) {
+            issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
+            umma_commit(s_full);
+            if (MODE == kSlice && (li + 2 >= ntiles || nx2.qk != nxt.qk)) umma_commit(q_empty);
+          }
         }
         // ---- dK(i) = dS Q, dQ += dS^T K
         wt(ds_full, li & 1, 0x50B);
@@ -304,13 +310,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (first_of_hp && hp > 0) wt(dq_empty, (hp - 1) & 1, 0x50D);
         if (!ok) break;
         tc_fence_after();
-        if (MODE == kFull) {
+        const bool last_of_hp = !more || newhead;
+        if (elect_one()) {
+          if (MODE == kFull) {
 #pragma unroll
-          for (int k = 0; k < PS / 16; ++k)
-            umma_ss(tmem + C::DK_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dQm, k * 2048),
-                    idTD, k > 0 ? 1u : 0u);
-        }
-        {
+            for (int k = 0; k < PS / 16; ++k)
+              umma_ss(tmem + C::DK_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dQm, k * 2048),
+                      idTD, k > 0 ? 1u : 0u);
+          }
           const uint64_t dKm = sdesc_add(dRm, uint32_t(sK) * C::KV_TILE);
 #pragma unroll
           for (int k = 0; k < T / 16; ++k)
@@ -318,15 +325,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int mb = 0; mb < PS / 128; ++mb)
               umma_ss(tmem + C::DQ_COL + mb * D, sdesc_add(dABm, mb * 2 * (T * 128) + k * 2048),
                       sdesc_add(dKm, k * 2048), idQD, (first_of_hp && k == 0) ? 0u : 1u);
+          umma_commit(ab_empty);
+          umma_commit(ring_empty(sK));
+          if (last_of_hp) {
+            umma_commit(dq_full);
+            if (MODE == kFull) umma_commit(q_empty);  // dK read Q up to here
+          }
         }
-        umma_commit(ab_empty);
-        umma_commit(ring_empty(sK));
-        const bool last_of_hp = !more || newhead;
-        if (last_of_hp) {
-          umma_commit(dq_full);
-          if (MODE == kFull) umma_commit(q_empty);  // dK read Q up to here
-          ++hp;
-        }
+        if (last_of_hp) ++hp;
         first_of_hp = last_of_hp;
         // ---- S(i+1) after a head change in full mode (Q replaced once dK(i) is done)
         if (more && !early) {
@@ -336,14 +342,16 @@ __global__ void __launch_bounds__(kThreads, 1)
           wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x510);
           if (!ok) break;
           tc_fence_after();
-          issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
-          umma_commit(s_full);
+          if (elect_one()) {
+            issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
+            umma_commit(s_full);
+          }
         }
         cur.next();
         nxt.next();
         nx2.next();
       }
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       mbar_wait_bounded(drain, 0, 200000000ull);
     } else if (warp == 2 || warp == 3) {
       // ------------------------------------ dsketch rows -> bf16, swizzled [d/64][PS][64]
@@ -684,7 +692,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
                                              __nv_bfloat16* __restrict__ dV) {
   using C = TokCfg<D, P>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (ws_failed(a.ws)) return;
   if (smem_u32(smem) & 1023u) {
     if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB21u);
@@ -795,7 +803,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
         for (int s = 0; s < C::NSLOT; ++s)
           if ((used >> s) & 1u) mbar_wait_bounded(full_bar(s), (par >> s) & 1u, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ---------------------------------------------------------- UMMA issuer
       // Per chunk g: dA_g, [dV | qbar]_g, S_{g+1}, u_g.  Shared-memory
       // descriptors are built once per operand and stepped by constant offsets,
@@ -806,7 +814,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
       bool ok = true;
       uint32_t fpar = 0u;  // per slot, as bits: parity of the next "full" phase
       auto wt = [&](uint32_t bar, uint32_t parity, uint32_t site) {
-        return ok = ok && mbar_wait(bar, parity, abort_flag, a.ws, site);
+        return ok = ok && mbar_wait_warp(bar, parity, abort_flag, a.ws, site);
       };
       auto wfull = [&](int s, uint32_t site) {
         wt(full_bar(s), (fpar >> s) & 1u, site);
@@ -830,7 +838,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
       wfull(2 * tok_qg_pair(0, 0) + 1, 0x902);
       if (ok) {
         tc_fence_after();
-        issue_S(0);
+        if (elect_one()) issue_S(0);
       }
       for (uint32_t g = 0; g < nchunks && ok; ++g) {
         const int li = int(g / C::NCH), c = int(g % C::NCH);
@@ -844,29 +852,29 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
         else if (g > 0) wt(sd_free_da, (g - 1) & 1, 0x905);
         if (!ok) break;
         tc_fence_after();
-        {
+        if (elect_one()) {
           const uint64_t dV = kmaj(slot_addr(2 * kvp + 1)), dG = kmaj(aG);
 #pragma unroll
           for (int k = 0; k < D / 16; ++k)
             umma_ss(tmem + tok_da_col<D, P, TW>(), sdesc_add(dV, kstep(k)), sdesc_add(dG, kstep(k)), idS,
                     k > 0 ? 1u : 0u);
+          umma_commit(da_full);
+          if (c == C::NCH - 1) umma_commit(empty_bar(2 * kvp + 1));  // last dA: V free
         }
-        umma_commit(da_full);
-        if (c == C::NCH - 1) umma_commit(empty_bar(2 * kvp + 1));  // last dA: V free
         // ---- [dV | qbar] += A [G_g | Q_g]
         wt(a_full, g & 1, 0x906);
         if (c == 0 && li > 0) wt(acc_empty, (li - 1) & 1, 0x907);
         if (!ok) break;
         tc_fence_after();
-        {
+        if (elect_one()) {
           const uint64_t dGQ = sdesc(aG, C::NC * 128, 1024);  // MN-major, 64-column blocks 16 KB apart
 #pragma unroll
           for (int k = 0; k < C::NC / 16; ++k)
             umma_ss(tmem + C::DV_COL, sdesc_add(dAB, kstep(k)), sdesc_add(dGQ, k * 2048), idGQ,
                     (c == 0 && k == 0) ? 0u : 1u);
+          umma_commit(ab_free_a);
+          umma_commit(empty_bar(2 * qgp));  // G chunk free
         }
-        umma_commit(ab_free_a);
-        umma_commit(empty_bar(2 * qgp));  // G chunk free
         // ---- S_{g+1}
         if (g + 1 < nchunks) {
           const uint32_t gn = g + 1;
@@ -876,24 +884,24 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
           wt(TW ? sd_free_s : sd_free_da, g & 1, 0x90A);  // S's columns read
           if (!ok) break;
           tc_fence_after();
-          issue_S(gn);
+          if (elect_one()) issue_S(gn);
         }
         // ---- u += E Q_g
         wt(e_full, g & 1, 0x90B);
         if (!ok) break;
         tc_fence_after();
-        {
+        if (elect_one()) {
           const uint64_t dQm = sdesc(aQ, C::NC * 128, 1024);
 #pragma unroll
           for (int k = 0; k < C::NC / 16; ++k)
             umma_ss(tmem + C::U_COL, sdesc_add(dAB, kstep(k)), sdesc_add(dQm, k * 2048), idU,
                     (c == 0 && k == 0) ? 0u : 1u);
+          umma_commit(ab_free_e);
+          umma_commit(empty_bar(2 * qgp + 1));  // Q chunk free
+          if (c == C::NCH - 1) umma_commit(acc_full);
         }
-        umma_commit(ab_free_e);
-        umma_commit(empty_bar(2 * qgp + 1));  // Q chunk free
-        if (c == C::NCH - 1) umma_commit(acc_full);
       }
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       mbar_wait_bounded(drain, 0, 200000000ull);
     }
   } else if (ntiles > 0) {
@@ -1276,7 +1284,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
                                             const float* __restrict__ lse, const float* __restrict__ Dco) {
   using C = QCfg<D, PS>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (ws_failed(a.ws)) return;
   if (smem_u32(smem) & 1023u) {
     if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB31u);
@@ -1385,7 +1393,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
           if (li + C::NV >= loaded) mbar_wait_bounded(ring_full(v_slot(li)), (li / C::NV) & 1, 200000000ull);
         }
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ---------------------------------------------------------- UMMA issuer
       // Order: S(0), dA(0);
       // then per tile i: S(i+1), dA(i+1), dQ(i), so the next tile's scores are
@@ -1400,7 +1408,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       int hc = 0, gc = 0, hp = 0;
       bool ok = true;
       auto wt = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return ok = ok && mbar_wait(bar, par, abort_flag, a.ws, site);
+        return ok = ok && mbar_wait_warp(bar, par, abort_flag, a.ws, site);
       };
       // waits for tile li's K and V, returns its control bits
       auto wait_kv = [&](int li) -> uint32_t {
@@ -1421,16 +1429,18 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
         tc_fence_after();
         const int sK = k_slot(li), sV = v_slot(li);
         const uint64_t dK = sdesc(sRing + sK * C::KV_TILE, 16, 1024), dV = sdesc(sRing + sV * C::KV_TILE, 16, 1024);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < D / 16; ++k)
-          umma_ss(tmem + C::S_COL, sdesc_add(dQs, step_p(k)), sdesc_add(dK, step_t(k)), idPT, k > 0 ? 1u : 0u);
+          for (int k = 0; k < D / 16; ++k)
+            umma_ss(tmem + C::S_COL, sdesc_add(dQs, step_p(k)), sdesc_add(dK, step_t(k)), idPT, k > 0 ? 1u : 0u);
 #pragma unroll
-        for (int k = 0; k < D / 16; ++k)  // G from TMEM: 8 columns (16 values of d) per step
-          umma_ts(tmem + C::DA_COL, tmem + C::G_COL + 8 * k, sdesc_add(dV, step_t(k)), idPT, k > 0 ? 1u : 0u);
-        umma_commit(sda_full);
-        umma_commit(ring_empty(sV));                // V read by its only product
-        if (fl & kHeadLast) umma_commit(q_empty);   // last S of this head piece
-        if (fl & kSegLast) umma_commit(g_empty);    // last dA of this segment
+          for (int k = 0; k < D / 16; ++k)  // G from TMEM: 8 columns (16 values of d) per step
+            umma_ts(tmem + C::DA_COL, tmem + C::G_COL + 8 * k, sdesc_add(dV, step_t(k)), idPT, k > 0 ? 1u : 0u);
+          umma_commit(sda_full);
+          umma_commit(ring_empty(sV));                // V read by its only product
+          if (fl & kHeadLast) umma_commit(q_empty);   // last S of this head piece
+          if (fl & kSegLast) umma_commit(g_empty);    // last dA of this segment
+        }
       };
       uint32_t fl_cur = wait_kv(0);
       if (ok) issue_sda(0, fl_cur);
@@ -1449,7 +1459,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
         if (first_of_hp && hp > 0) wt(dq_empty, (hp - 1) & 1, 0xD0A);
         if (!ok) break;
         tc_fence_after();
-        {
+        if (elect_one()) {
           const int sK = k_slot(li);
           const uint64_t dK = sdesc(sRing + sK * C::KV_TILE, T * 128, 1024);  // MN-major: d blocks 16 KB apart
           const uint32_t dsb = tmem + C::DS_COL;
@@ -1462,7 +1472,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
         if (fl_cur & kHeadLast) ++hp;
         fl_cur = fl_next;
       }
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       mbar_wait_bounded(drain, 0, 200000000ull);
     } else if (warp == 2 || warp == 3) {
       // ------------------------------------------------- per-token columns

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   float* __restrict__ lse_out, const float* __restrict__ lse_in) {
   using C = Cfg<D, PS, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   constexpr bool PAIR = (MODE == kPair);
   // A pair's CTAs must both reach the cluster barriers below, so pair mode
   // never returns early: a failed call or a misaligned base only skips work.
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
         if (hc > 0) mbar_wait_bounded(q_full, uint32_t(hc - 1) & 1u, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ------------------------------------------------------ UMMA issuer
       constexpr uint32_t idS = idesc_bf16(128, PS, 0, 0);
       constexpr uint32_t idO = C::TRANS ? idesc_bf16(128, PS, 1, 1) : idesc_bf16(128, D, 1, 1);
@@ -240,8 +240,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       // under a test limit (sa_set_wait_limit_ns) the issuer first waits for a
       // barrier nothing completes: the limit runs out and the CTA takes its
       // abort path (drains, TMEM freed, SA_ERR_TIMEOUT)
-      bool ok = ctl_wait_limit(abort_flag) >= kPollLimitNs || mbar_wait(never, 0, abort_flag, a.ws, 0x200);
-      ok = ok && mbar_wait(q_full, 0, abort_flag, a.ws, 0x201);
+      bool ok = ctl_wait_limit(abort_flag) >= kPollLimitNs || mbar_wait_warp(never, 0, abort_flag, a.ws, 0x200);
+      ok = ok && mbar_wait_warp(q_full, 0, abort_flag, a.ws, 0x201);
       // operand descriptors built once and stepped by constant offsets: the
       // issuing thread shares its sub-partition with two softmax warps, and each
       // instruction it saves shortens the issue of a group
@@ -255,13 +255,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                   sdesc_add(dQ0, (k >> 2) * (PS * 128) + (k & 3) * 32), idS, k > 0 ? 1u : 0u);
       };
       if (ok) {
-        ok = mbar_wait(ring_full(0), 0, abort_flag, a.ws, 0x202);
+        ok = mbar_wait_warp(ring_full(0), 0, abort_flag, a.ws, 0x202);
         if (ok) {
           tc_fence_after();
-          issue_S(0);
-          umma_commit(s_full);
-          umma_commit(ring_empty(0));
-          if (ntiles == 1 || nxt.qk != cur.qk) umma_commit(q_empty);
+          if (elect_one()) {
+            issue_S(0);
+            umma_commit(s_full);
+            umma_commit(ring_empty(0));
+            if (ntiles == 1 || nxt.qk != cur.qk) umma_commit(q_empty);
+          }
           e = 1;
         }
       }
@@ -269,65 +271,67 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (li + 1 < ntiles) {
           if (nxt.qk != cur.qk) {
             ++hc;
-            ok = mbar_wait(q_full, hc & 1, abort_flag, a.ws, 0x203);
+            ok = mbar_wait_warp(q_full, hc & 1, abort_flag, a.ws, 0x203);
             if (!ok) break;
           }
-          ok = mbar_wait(s_empty, li & 1, abort_flag, a.ws, 0x204);
+          ok = mbar_wait_warp(s_empty, li & 1, abort_flag, a.ws, 0x204);
           if (!ok) break;
           const int s = int(e % C::NSLOT);
-          ok = mbar_wait(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x205);
+          ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x205);
           if (!ok) break;
           tc_fence_after();
-          issue_S(uint32_t(s));
-          umma_commit(s_full);
-          umma_commit(ring_empty(s));
+          if (elect_one()) {
+            issue_S(uint32_t(s));
+            umma_commit(s_full);
+            umma_commit(ring_empty(s));
+          }
           ++e;
           // last S of these prototypes: Q may be replaced once it completes
           const int q_now = nxt.qk;
           nxt.next();
-          if (li + 2 >= ntiles || nxt.qk != q_now) umma_commit(q_empty);
+          if ((li + 2 >= ntiles || nxt.qk != q_now) && elect_one()) umma_commit(q_empty);
         }
         // aggregation of tile li
-        ok = mbar_wait(w_full, li & 1, abort_flag, a.ws, 0x206);
+        ok = mbar_wait_warp(w_full, li & 1, abort_flag, a.ws, 0x206);
         if (!ok) break;
         const int s = int(e % C::NSLOT);
-        ok = mbar_wait(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x207);
+        ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x207);
         if (!ok) break;
         // segment sc accumulates into buffer sc % NOB, free once the softmax
         // warps have stored the segment that used it last
         const int ob = sc % C::NOB;
         if (cur.seg_first && sc >= C::NOB) {
-          ok = mbar_wait(o_empty_of(ob), uint32_t((sc / C::NOB) - 1) & 1u, abort_flag, a.ws, 0x208);
+          ok = mbar_wait_warp(o_empty_of(ob), uint32_t((sc / C::NOB) - 1) & 1u, abort_flag, a.ws, 0x208);
           if (!ok) break;
         }
         tc_fence_after();
         const uint64_t dV = sdesc_add(dV0, uint32_t(s) * C::KV_TILE);
         const uint32_t ocol = tmem + C::O_COL + uint32_t(ob * C::O_COLS);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < T / 16; ++k) {
-          const uint32_t acc = (cur.seg_first && k == 0) ? 0u : 1u;
-          if (C::TRANS) {
-            // O^T[d, p] += sum_t V[t, d] A[t, p]:  A-operand V^T (MN-major), B-operand A (MN-major)
-            umma_ss(ocol, sdesc_add(dV, k * 2048), sdesc_add(dW0, k * 2048), idO, acc);
-          } else {
+          for (int k = 0; k < T / 16; ++k) {
+            const uint32_t acc = (cur.seg_first && k == 0) ? 0u : 1u;
+            if (C::TRANS) {
+              // O^T[d, p] += sum_t V[t, d] A[t, p]:  A-operand V^T (MN-major), B-operand A (MN-major)
+              umma_ss(ocol, sdesc_add(dV, k * 2048), sdesc_add(dW0, k * 2048), idO, acc);
+            } else {
 #pragma unroll
-            for (int mb = 0; mb < PS / 128; ++mb)
-              // O[p, d] += sum_t A[t, p] V[t, d]: A-operand A^T (MN-major), B-operand V (MN-major)
-              umma_ss(ocol + mb * D, sdesc_add(dW0, mb * 2 * (T * 128) + k * 2048), sdesc_add(dV, k * 2048), idO,
-                      acc);
+              for (int mb = 0; mb < PS / 128; ++mb)
+                // O[p, d] += sum_t A[t, p] V[t, d]: A-operand A^T (MN-major), B-operand V (MN-major)
+                umma_ss(ocol + mb * D, sdesc_add(dW0, mb * 2 * (T * 128) + k * 2048), sdesc_add(dV, k * 2048), idO,
+                        acc);
+            }
           }
+          umma_commit(w_empty);
+          umma_commit(ring_empty(s));
+          if (cur.seg_last) umma_commit(o_full_of(ob));
         }
-        umma_commit(w_empty);
-        umma_commit(ring_empty(s));
         ++e;
-        if (cur.seg_last) {
-          umma_commit(o_full_of(ob));
-          ++sc;
-        }
+        if (cur.seg_last) ++sc;
         cur.next();
       }
       // make sure no UMMA is still running when TMEM is released
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       mbar_wait_bounded(drain, 0, 200000000ull);
     }
   } else if (ntiles > 0) {
@@ -540,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   float* __restrict__ lse_out, float2* __restrict__ part_out) {
   using C = LseCfg<D, NC, NCH>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (ws_failed(a.ws)) return;
   if (smem_u32(smem) & 1023u) {
     if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xA12u);
@@ -620,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (uint32_t k = (e > uint32_t(C::NSLOT) ? e - C::NSLOT : 0); k < e; ++k)
           mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       constexpr uint32_t idS = idesc_bf16(128, NC, 0, 0);
       TileWalker cur(a, tb, te, T);
       int hc = 0, prev_h = -1;
@@ -630,33 +634,37 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int h_now = cur.qk;
         if (h_now != prev_h) {
           prev_h = h_now;
-          ok = mbar_wait(q_full, hc & 1, abort_flag, a.ws, 0x211);
+          ok = mbar_wait_warp(q_full, hc & 1, abort_flag, a.ws, 0x211);
           ++hc;
           if (!ok) break;
         }
         const int s = int(uint32_t(li) % C::NSLOT);
-        ok = mbar_wait(ring_full(s), (uint32_t(li) / C::NSLOT) & 1, abort_flag, a.ws, 0x212);
+        ok = mbar_wait_warp(ring_full(s), (uint32_t(li) / C::NSLOT) & 1, abort_flag, a.ws, 0x212);
         if (!ok) break;
         const uint32_t kaddr = sRing + s * C::KV_TILE;
         for (int c = 0; c < NCH && ok; ++c, ++g) {
           const int buf = int(g & 1);
-          if (g >= 2) ok = mbar_wait(s_empty0 + 8 * buf, ((g >> 1) + 1) & 1, abort_flag, a.ws, 0x213);
+          if (g >= 2) ok = mbar_wait_warp(s_empty0 + 8 * buf, ((g >> 1) + 1) & 1, abort_flag, a.ws, 0x213);
           if (!ok) break;
           tc_fence_after();
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) {
-            const uint64_t ad = sdesc(kaddr + (k >> 2) * (T * 128) + (k & 3) * 32, 16, 1024);
-            const uint64_t bd = sdesc(sQ + (k >> 2) * (C::P * 128) + c * NC * 128 + (k & 3) * 32, 16, 1024);
-            umma_ss(tmem + buf * NC, ad, bd, idS, k > 0 ? 1u : 0u);
+            for (int k = 0; k < D / 16; ++k) {
+              const uint64_t ad = sdesc(kaddr + (k >> 2) * (T * 128) + (k & 3) * 32, 16, 1024);
+              const uint64_t bd = sdesc(sQ + (k >> 2) * (C::P * 128) + c * NC * 128 + (k & 3) * 32, 16, 1024);
+              umma_ss(tmem + buf * NC, ad, bd, idS, k > 0 ? 1u : 0u);
+            }
+            umma_commit(s_full0 + 8 * buf);
           }
-          umma_commit(s_full0 + 8 * buf);
         }
         if (!ok) break;
-        umma_commit(ring_empty(s));
         cur.next();
-        if (li + 1 >= ntiles || cur.qk != h_now) umma_commit(q_empty);
+        if (elect_one()) {
+          umma_commit(ring_empty(s));
+          if (li + 1 >= ntiles || cur.qk != h_now) umma_commit(q_empty);
+        }
       }
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       mbar_wait_bounded(drain, 0, 200000000ull);
     } else if (warp >= kSoftWarp0) {
       const int sw = (warp - kSoftWarp0) >> 2, q = warp & 3, row = 32 * q + lane;

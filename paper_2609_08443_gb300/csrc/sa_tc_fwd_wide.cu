@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
                        float* __restrict__ lse_out) {
   using C = WCfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // Both CTAs of a pair must reach the cluster barriers below, so a failed
   // call or a misaligned base only skips the work.
   bool skip = ws_failed(a.ws);
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         for (int li = (loaded > C::NV ? loaded - C::NV : 0); li < loaded; ++li)
           mbar_wait_bounded(vfull(li % C::NV), uint32_t(li / C::NV) & 1u, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ---------------------------------------------------------- UMMA issuer
       // Order: S(0); then per tile i: S(i+1) once the softmax warps hold S(i)
       // in registers, O(i) once the weights of tile i are stored.
@@ -262,9 +262,9 @@ __global__ void __launch_bounds__(kWThreads, 1)
       // under a test limit (sa_set_wait_limit_ns) the issuer first waits for a
       // barrier nothing completes: the limit runs out and the CTA takes its
       // abort path (drains, TMEM freed, SA_ERR_TIMEOUT)
-      bool ok = ctl_wait_limit(abort_flag) >= kPollLimitNs || mbar_wait(never, 0, abort_flag, a.ws, 0x220);
+      bool ok = ctl_wait_limit(abort_flag) >= kPollLimitNs || mbar_wait_warp(never, 0, abort_flag, a.ws, 0x220);
       auto wt = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return ok = ok && mbar_wait(bar, par, abort_flag, a.ws, site);
+        return ok = ok && mbar_wait_warp(bar, par, abort_flag, a.ws, site);
       };
       auto issue_S = [&](int li) {  // ws_ is at tile li
         if (ws_.qk != prev_q) {
@@ -276,19 +276,21 @@ __global__ void __launch_bounds__(kWThreads, 1)
         wt(kfull(s), uint32_t(li / C::NK) & 1u, 0x222);
         if (!ok) return;
         tc_fence_after();
-        const uint32_t kaddr = sK + s * C::KV_TILE;
+        if (elect_one()) {
+          const uint32_t kaddr = sK + s * C::KV_TILE;
 #pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint64_t ad = sdesc(kaddr + (k >> 2) * (T * 128) + (k & 3) * 32, 16, 1024);
-          const uint64_t bd = sdesc(sQ + (k >> 2) * (C::PS * 128) + (k & 3) * 32, 16, 1024);
-          umma_ss(tmem + C::S_COL, ad, bd, idS, k > 0 ? 1u : 0u);
+          for (int k = 0; k < D / 16; ++k) {
+            const uint64_t ad = sdesc(kaddr + (k >> 2) * (T * 128) + (k & 3) * 32, 16, 1024);
+            const uint64_t bd = sdesc(sQ + (k >> 2) * (C::PS * 128) + (k & 3) * 32, 16, 1024);
+            umma_ss(tmem + C::S_COL, ad, bd, idS, k > 0 ? 1u : 0u);
+          }
+          umma_commit(s_full);
+          umma_commit(kempty(s));
         }
-        umma_commit(s_full);
-        umma_commit(kempty(s));
         int64_t t0n;
         int nn, hn, qn;
         ws_.peek_next(t0n, nn, hn, qn);
-        if (li + 1 >= ntiles || qn != ws_.qk) umma_commit(q_empty);  // last S of these prototypes
+        if ((li + 1 >= ntiles || qn != ws_.qk) && elect_one()) umma_commit(q_empty);  // last S of these prototypes
         ws_.next();
       };
       auto issue_O = [&](int li) {  // wo is at tile li
@@ -298,28 +300,28 @@ __global__ void __launch_bounds__(kWThreads, 1)
         if (wo.seg_first && sc > 0) wt(o_empty, uint32_t(sc - 1) & 1u, 0x225);
         if (!ok) return;
         tc_fence_after();
-        const uint32_t vaddr = sV + s * C::KV_TILE;
+        if (elect_one()) {
+          const uint32_t vaddr = sV + s * C::KV_TILE;
 #pragma unroll
-        for (int k = 0; k < T / 16; ++k) {
-          const uint32_t acc = (wo.seg_first && k == 0) ? 0u : 1u;
-          if (C::TRANS) {
-            // O^T[d, p] += sum_t V[t, d] A[t, p]: A-operand V^T (MN-major), B-operand A (MN-major)
-            umma_ss(tmem + C::O_COL, sdesc(vaddr + k * 2048, T * 128, 1024), sdesc(sW + k * 2048, T * 128, 1024),
-                    idO, acc);
-          } else {
+          for (int k = 0; k < T / 16; ++k) {
+            const uint32_t acc = (wo.seg_first && k == 0) ? 0u : 1u;
+            if (C::TRANS) {
+              // O^T[d, p] += sum_t V[t, d] A[t, p]: A-operand V^T (MN-major), B-operand A (MN-major)
+              umma_ss(tmem + C::O_COL, sdesc(vaddr + k * 2048, T * 128, 1024), sdesc(sW + k * 2048, T * 128, 1024),
+                      idO, acc);
+            } else {
 #pragma unroll
-            for (int mb = 0; mb < C::PS / 128; ++mb)
-              // O[p, d] += sum_t A[t, p] V[t, d]: A-operand A^T (MN-major), B-operand V (MN-major)
-              umma_ss(tmem + C::O_COL + mb * D, sdesc(sW + mb * 2 * (T * 128) + k * 2048, T * 128, 1024),
-                      sdesc(vaddr + k * 2048, T * 128, 1024), idO, acc);
+              for (int mb = 0; mb < C::PS / 128; ++mb)
+                // O[p, d] += sum_t A[t, p] V[t, d]: A-operand A^T (MN-major), B-operand V (MN-major)
+                umma_ss(tmem + C::O_COL + mb * D, sdesc(sW + mb * 2 * (T * 128) + k * 2048, T * 128, 1024),
+                        sdesc(vaddr + k * 2048, T * 128, 1024), idO, acc);
+            }
           }
+          umma_commit(w_empty);
+          umma_commit(vempty(s));
+          if (wo.seg_last) umma_commit(o_full);
         }
-        umma_commit(w_empty);
-        umma_commit(vempty(s));
-        if (wo.seg_last) {
-          umma_commit(o_full);
-          ++sc;
-        }
+        if (wo.seg_last) ++sc;
         wo.next();
       };
       issue_S(0);
@@ -330,7 +332,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         }
         if (ok) issue_O(li);
       }
-      umma_commit(drain);  // no UMMA may still run when TMEM is released
+      if (elect_one()) umma_commit(drain);  // no UMMA may still run when TMEM is released
       mbar_wait_bounded(drain, 0, 200000000ull);
     }
   } else if (ntiles > 0) {

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      float* __restrict__ lse_tok, float2* __restrict__ stat_part) {
   using C = Cfg<D, NM>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (ws_failed(a.ws)) return;
   if (smem_u32(smem) & 1023u) {  // 128-byte swizzle atoms need 1024-byte alignment
     if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xA21u);
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (uint32_t k = (e > uint32_t(C::NSLOT) ? e - C::NSLOT : 0); k < e; ++k)
           mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ------------------------------------------------------ UMMA issuer
       constexpr uint32_t idS = idesc_bf16(128, T, 0, 0);  // Q (K-major) x K^T (K-major)
       constexpr uint32_t idO = idesc_bf16(128, D, 0, 1);  // A (K-major) x V (MN-major)
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       nxt.next();
       uint32_t e = 0;
       int hc = 0, sc = 0;
-      bool ok = mbar_wait(q_full, 0, abort_flag, a.ws, 0xA01);
+      bool ok = mbar_wait_warp(q_full, 0, abort_flag, a.ws, 0xA01);
       // S[m-tile] = Q[m-tile] K^T over the d features, 16 per step
       auto issue_S = [&](uint32_t slot) {
         const uint32_t kaddr = sRing + slot * C::KV_TILE;
@@ -200,13 +200,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       };
       if (ok) {
-        ok = mbar_wait(ring_full(0), 0, abort_flag, a.ws, 0xA02);
+        ok = mbar_wait_warp(ring_full(0), 0, abort_flag, a.ws, 0xA02);
         if (ok) {
           tc_fence_after();
-          issue_S(0);
-          umma_commit(s_full);
-          umma_commit(ring_empty(0));
-          if (ntiles == 1 || nxt.qk != cur.qk) umma_commit(q_empty);
+          if (elect_one()) {
+            issue_S(0);
+            umma_commit(s_full);
+            umma_commit(ring_empty(0));
+            if (ntiles == 1 || nxt.qk != cur.qk) umma_commit(q_empty);
+          }
           e = 1;
         }
       }
@@ -214,55 +216,57 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (li + 1 < ntiles) {
           if (nxt.qk != cur.qk) {
             ++hc;
-            ok = mbar_wait(q_full, hc & 1, abort_flag, a.ws, 0xA03);
+            ok = mbar_wait_warp(q_full, hc & 1, abort_flag, a.ws, 0xA03);
             if (!ok) break;
           }
-          ok = mbar_wait(s_empty, li & 1, abort_flag, a.ws, 0xA04);
+          ok = mbar_wait_warp(s_empty, li & 1, abort_flag, a.ws, 0xA04);
           if (!ok) break;
           const int s = int(e % C::NSLOT);
-          ok = mbar_wait(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA05);
+          ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA05);
           if (!ok) break;
           tc_fence_after();
-          issue_S(uint32_t(s));
-          umma_commit(s_full);
-          umma_commit(ring_empty(s));
+          if (elect_one()) {
+            issue_S(uint32_t(s));
+            umma_commit(s_full);
+            umma_commit(ring_empty(s));
+          }
           ++e;
           const int q_now = nxt.qk;
           nxt.next();
-          if (li + 2 >= ntiles || nxt.qk != q_now) umma_commit(q_empty);
+          if ((li + 2 >= ntiles || nxt.qk != q_now) && elect_one()) umma_commit(q_empty);
         }
         // O[m-tile] += A[m-tile] V over the tile's 128 tokens, 16 per step
-        ok = mbar_wait(w_full, li & 1, abort_flag, a.ws, 0xA06);
+        ok = mbar_wait_warp(w_full, li & 1, abort_flag, a.ws, 0xA06);
         if (!ok) break;
         const int s = int(e % C::NSLOT);
-        ok = mbar_wait(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA07);
+        ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA07);
         if (!ok) break;
         if (cur.seg_first && sc > 0) {
-          ok = mbar_wait(o_empty, (sc - 1) & 1, abort_flag, a.ws, 0xA08);
+          ok = mbar_wait_warp(o_empty, (sc - 1) & 1, abort_flag, a.ws, 0xA08);
           if (!ok) break;
         }
         tc_fence_after();
-        const uint32_t vaddr = sRing + s * C::KV_TILE;
+        if (elect_one()) {
+          const uint32_t vaddr = sRing + s * C::KV_TILE;
 #pragma unroll
-        for (int k = 0; k < T / 16; ++k) {
-          const uint32_t acc = (cur.seg_first && k == 0) ? 0u : 1u;
+          for (int k = 0; k < T / 16; ++k) {
+            const uint32_t acc = (cur.seg_first && k == 0) ? 0u : 1u;
 #pragma unroll
-          for (int mt = 0; mt < NM; ++mt) {
-            const uint64_t ad = sdesc(sW + (k >> 2) * (C::PS * 128) + mt * (128 * 128) + (k & 3) * 32, 16, 1024);
-            const uint64_t bd = sdesc(vaddr + k * 2048, T * 128, 1024);
-            umma_ss(tmem + C::O_COL + mt * D, ad, bd, idO, acc);
+            for (int mt = 0; mt < NM; ++mt) {
+              const uint64_t ad = sdesc(sW + (k >> 2) * (C::PS * 128) + mt * (128 * 128) + (k & 3) * 32, 16, 1024);
+              const uint64_t bd = sdesc(vaddr + k * 2048, T * 128, 1024);
+              umma_ss(tmem + C::O_COL + mt * D, ad, bd, idO, acc);
+            }
           }
+          umma_commit(w_empty);
+          umma_commit(ring_empty(s));
+          if (cur.seg_last) umma_commit(o_full);
         }
-        umma_commit(w_empty);
-        umma_commit(ring_empty(s));
         ++e;
-        if (cur.seg_last) {
-          umma_commit(o_full);
-          ++sc;
-        }
+        if (cur.seg_last) ++sc;
         cur.next();
       }
-      umma_commit(drain);  // no UMMA may still run when TMEM is released
+      if (elect_one()) umma_commit(drain);  // no UMMA may still run when TMEM is released
       mbar_wait_bounded(drain, 0, 200000000ull);
     }
   } else if (ntiles > 0) {
