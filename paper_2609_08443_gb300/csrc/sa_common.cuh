@@ -8,8 +8,8 @@
 // gets the same number of tiles to within one.  A (user, head) segment that
 // falls entirely inside one worker's range is finished by that worker; a
 // segment cut by range boundaries leaves one fp32 partial per worker, and a
-// finalize kernel adds them in worker order, which makes the result bitwise
-// reproducible for a given W.
+// finalize kernel adds them in an order fixed by the plan, which makes the
+// result bitwise reproducible for a given W.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -24,6 +24,7 @@ namespace sa {
 constexpr int kMaxP = 2048;
 constexpr int kMaxD = 128;
 constexpr int kMaxH = 64;
+constexpr int kMaxWorkers = 1024;  // workers of a plan (3 per SM at most: 456 on a 152-SM GB300)
 
 // ---------------------------------------------------------------- workspace
 struct WsHeader {

@@ -32,7 +32,7 @@ SA_HD int q_row(const Args& a, int b, int h) { return a.uq ? b * a.H + h : h; }
 // (sa_set_wait_limit_ns; the planner copies it into each call's workspace).
 uint64_t wait_limit_ns();
 
-// planner / finalize (sa_simt.cu)
+// planner (sa_simt.cu), finalize (sa_finalize.cu)
 cudaError_t launch_plan(const Args& a, int T, cudaStream_t st);
 cudaError_t launch_finalize_sketch(const Args& a, int W, float* sketch, cudaStream_t st);
 cudaError_t launch_finalize_dq(const Args& a, int W, float* dQ, cudaStream_t st);

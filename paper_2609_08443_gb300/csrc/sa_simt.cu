@@ -1,6 +1,6 @@
-// CUDA-core kernels of the SA sketching step: the ragged planner, the
-// fixed-order finalize reductions, and a fp32-arithmetic path used for fp32
-// inputs and for shapes the tensor-core kernels do not cover.
+// CUDA-core kernels of the SA sketching step: the ragged planner and a
+// fp32-arithmetic path used for fp32 inputs and for shapes the tensor-core
+// kernels do not cover.
 //
 // Forward (paper Sec. 3.1): per token the log-sum-exp over the P prototypes is
 // computed first (sa_simt_lse), then blocks of 64 prototypes accumulate
@@ -68,106 +68,6 @@ __global__ void __launch_bounds__(1024) plan_kernel(const int32_t* __restrict__ 
     prefix[B] = carry;
     ws_header(ws)->tiles_per_head = carry;
     ws_header(ws)->err = bad ? uint32_t(SA_ERR_BAD_SEQLENS) : 0u;
-  }
-}
-
-// out[e] (+)= sum over k < n of src[off[k] + e] for e < PD, in k order; the
-// first chunk of workers starts from zero, later chunks continue the running
-// sum held in out (so the rounding is that of one sum in worker order).  A
-// negative off[k] is a worker with an empty range.  float4 accesses when every
-// address is 16-byte aligned.
-__device__ __forceinline__ void sum_pieces(const float* __restrict__ src, const int64_t* off, int n,
-                                           bool first, int64_t PD, float* __restrict__ out, int64_t e0,
-                                           int64_t estep) {
-  bool vec = (PD & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
-  if (vec) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    float4* o4 = reinterpret_cast<float4*>(out);
-    for (int64_t e = e0; e < PD / 4; e += estep) {
-      float4 s = first ? make_float4(0.f, 0.f, 0.f, 0.f) : o4[e];
-      for (int k = 0; k < n; ++k) {
-        if (off[k] < 0) continue;
-        const float4 v = s4[off[k] / 4 + e];
-        s.x += v.x;
-        s.y += v.y;
-        s.z += v.z;
-        s.w += v.w;
-      }
-      o4[e] = s;
-    }
-    return;
-  }
-  for (int64_t e = e0; e < PD; e += estep) {
-    float s = first ? 0.f : out[e];
-    for (int k = 0; k < n; ++k)
-      if (off[k] >= 0) s += src[off[k] + e];
-    out[e] = s;
-  }
-}
-
-// Sum of the pieces of every cut (user, head) segment, in worker order; zero
-// sketch for empty users.  grid = B*H blocks.  The pieces' offsets are found
-// once per block (range_begin divides in 64 bits), then summed element-wise.
-__global__ void __launch_bounds__(256) finalize_sketch_kernel(const void* ws, const int64_t* prefix,
-                                                              int B, int H, int P, int d, int W,
-                                                              const float* __restrict__ partial,
-                                                              float* __restrict__ sketch) {
-  __shared__ int64_t off[256];
-  if (ws_failed(ws)) return;
-  const int64_t tph = reinterpret_cast<const WsHeader*>(ws)->tiles_per_head;
-  const int64_t total = tph * H;
-  const int bh = blockIdx.x, b = bh / H, h = bh % H;
-  const int64_t seg0 = int64_t(h) * tph + prefix[b], seg1 = int64_t(h) * tph + prefix[b + 1];
-  const int64_t PD = int64_t(P) * d;
-  float* out = sketch + int64_t(bh) * PD;
-  if (seg0 == seg1) {
-    for (int64_t e = threadIdx.x; e < PD; e += blockDim.x) out[e] = 0.f;
-    return;
-  }
-  const int g0 = owner_of(total, W, seg0), g1 = owner_of(total, W, seg1 - 1);
-  if (g0 == g1) return;  // written whole by its worker
-  for (int c0 = g0; c0 <= g1; c0 += 256) {
-    const int n = min(256, g1 - c0 + 1);
-    __syncthreads();
-    if (int(threadIdx.x) < n) {
-      const int g = c0 + int(threadIdx.x);
-      off[threadIdx.x] = range_begin(total, W, g) == range_begin(total, W, g + 1)
-                             ? int64_t(-1)
-                             : (int64_t(g) * 2 + partial_slot(total, W, g, seg0)) * PD;
-    }
-    __syncthreads();
-    sum_pieces(partial, off, n, c0 == g0, PD, out, threadIdx.x, blockDim.x);
-  }
-}
-
-// dQ[h] = sum over the workers whose range meets head h of their partial.
-__global__ void __launch_bounds__(256) finalize_dq_kernel(const void* ws, int H, int P, int d, int W,
-                                                          const float* __restrict__ dq_partial,
-                                                          float* __restrict__ dQ) {
-  __shared__ int64_t off[256];
-  if (ws_failed(ws)) return;
-  const int64_t tph = reinterpret_cast<const WsHeader*>(ws)->tiles_per_head;
-  const int64_t total = tph * H;
-  const int h = blockIdx.y;
-  const int64_t PD = int64_t(P) * d;
-  float* out = dQ + int64_t(h) * PD;
-  const int64_t e0 = blockIdx.x * int64_t(blockDim.x) + threadIdx.x, stride = int64_t(gridDim.x) * blockDim.x;
-  if (tph == 0) {
-    for (int64_t e = e0; e < PD; e += stride) out[e] = 0.f;
-    return;
-  }
-  const int g0 = owner_of(total, W, int64_t(h) * tph), g1 = owner_of(total, W, int64_t(h + 1) * tph - 1);
-  for (int c0 = g0; c0 <= g1; c0 += 256) {
-    const int n = min(256, g1 - c0 + 1);
-    __syncthreads();
-    if (int(threadIdx.x) < n) {
-      const int g = c0 + int(threadIdx.x);
-      off[threadIdx.x] = range_begin(total, W, g) == range_begin(total, W, g + 1)
-                             ? int64_t(-1)
-                             : (int64_t(g) * H + h) * PD;
-    }
-    __syncthreads();
-    sum_pieces(dq_partial, off, n, c0 == g0, PD, out, e0, stride);
   }
 }
 
@@ -546,18 +446,6 @@ cudaError_t launch_plan(const Args& a, int T, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize_sketch(const Args& a, int W, float* sketch, cudaStream_t st) {
-  if (a.B * int64_t(a.H) == 0) return cudaSuccess;
-  finalize_sketch_kernel<<<a.B * a.H, 256, 0, st>>>(a.ws, a.prefix, a.B, a.H, a.P, a.d, W, a.partial, sketch);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_finalize_dq(const Args& a, int W, float* dQ, cudaStream_t st) {
-  dim3 grid(32, a.H);
-  finalize_dq_kernel<<<grid, 256, 0, st>>>(a.ws, a.H, a.P, a.d, W, a.dq_partial, dQ);
-  return cudaGetLastError();
-}
-
 template <typename T>
 static cudaError_t set_smem(const void* fn, size_t bytes) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
@@ -635,7 +523,7 @@ int simt_tile_tokens() { return ST; }
 int simt_workers(int num_sms, int P) {
   const int nb = (P + SPB - 1) / SPB;
   int w = (3 * num_sms + nb - 1) / nb;
-  return w < 1 ? 1 : w;
+  return w < 1 ? 1 : w > kMaxWorkers ? kMaxWorkers : w;
 }
 
 }  // namespace sa

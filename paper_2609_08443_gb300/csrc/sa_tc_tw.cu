@@ -17,7 +17,7 @@
 // the thread's row of O rescaled in TMEM (after the previous aggregation has
 // completed, before the next is issued).  A user's sketch is normalised by the
 // sum when its segment ends; a worker's piece of a segment cut across workers
-// is left unnormalised with its (shift, sum) for tw_finalize_kernel.
+// is left unnormalised with its (shift, sum) for launch_tw_finalize.
 //
 // One CTA holds PS = 128 NM prototypes (grid.y = P / PS slices); warpgroup g of
 // the softmax warps owns M-tile g.  Warp roles: 0 = TMA producer, 1 = UMMA

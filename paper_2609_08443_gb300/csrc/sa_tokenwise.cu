@@ -9,7 +9,7 @@
 // the P prototypes as queries) and rescales its accumulator when m_j grows.  A
 // worker that holds a whole (user, head) segment writes O_j = acc_j / l_j and
 // lse_j = m_j + log l_j; a cut segment leaves (acc_j, m_j, l_j) per worker, and
-// tw_finalize merges those in worker order (bitwise reproducible).
+// launch_tw_finalize merges those in a fixed order (bitwise reproducible).
 //
 // Backward (chain rule; the paper prints none), with G = dsketch[b, h]:
 //     dV_i = sum_j A[j,i] G_j,    D_j = sum_i A[j,i] (G_j . v_i) = G_j . O_j,
@@ -135,49 +135,6 @@ __global__ void __launch_bounds__(TNT) tw_fwd_kernel(Args a, float* __restrict__
       m = -INFINITY;
       l = 0.f;
     }
-  }
-}
-
-// Merge of the pieces of every cut (user, head) segment in worker order:
-// M = max_g m_g, L = sum_g l_g e^(m_g - M), O = sum_g acc_g e^(m_g - M) / L,
-// lse = M + log L.  Empty users: zero sketch and lse = -inf.  grid = B*H.
-__global__ void __launch_bounds__(256) tw_finalize_kernel(const void* ws, const int64_t* prefix, int B, int H,
-                                                          int P, int d, int W, const float* __restrict__ partial,
-                                                          const float2* __restrict__ stat_part,
-                                                          float* __restrict__ sketch, float* __restrict__ lse_tok) {
-  if (ws_failed(ws)) return;
-  const int64_t tph = reinterpret_cast<const WsHeader*>(ws)->tiles_per_head;
-  const int64_t total = tph * H;
-  const int bh = blockIdx.x, b = bh / H, h = bh % H;
-  const int64_t seg0 = int64_t(h) * tph + prefix[b], seg1 = int64_t(h) * tph + prefix[b + 1];
-  const int64_t PD = int64_t(P) * d;
-  float* out = sketch + int64_t(bh) * PD;
-  if (seg0 == seg1) {
-    for (int64_t e = threadIdx.x; e < PD; e += blockDim.x) out[e] = 0.f;
-    for (int j = threadIdx.x; j < P; j += blockDim.x) lse_tok[int64_t(bh) * P + j] = -INFINITY;
-    return;
-  }
-  const int g0 = owner_of(total, W, seg0), g1 = owner_of(total, W, seg1 - 1);
-  if (g0 == g1) return;  // written whole by its worker
-  for (int64_t e = threadIdx.x; e < PD; e += blockDim.x) {
-    const int j = int(e / d);
-    float M = -INFINITY;
-    for (int g = g0; g <= g1; ++g) {
-      if (range_begin(total, W, g) == range_begin(total, W, g + 1)) continue;
-      const int64_t slot = int64_t(g) * 2 + partial_slot(total, W, g, seg0);
-      M = fmaxf(M, stat_part[slot * P + j].x);
-    }
-    float L = 0.f, o = 0.f;
-    for (int g = g0; g <= g1; ++g) {
-      if (range_begin(total, W, g) == range_begin(total, W, g + 1)) continue;
-      const int64_t slot = int64_t(g) * 2 + partial_slot(total, W, g, seg0);
-      const float2 st = stat_part[slot * P + j];
-      const float f = expf(st.x - M);
-      L = fmaf(st.y, f, L);
-      o = fmaf(partial[slot * PD + e], f, o);
-    }
-    out[e] = o / L;
-    if (e - int64_t(j) * d == 0) lse_tok[int64_t(bh) * P + j] = M + logf(L);
   }
 }
 
@@ -406,13 +363,6 @@ cudaError_t launch_tw_fwd(const Args& a, int W, float* sketch, float* lse_tok, f
   const dim3 grid(W, (a.P + TPB - 1) / TPB);
   if (a.dt == SA_BF16) return run(&tw_fwd_kernel<__nv_bfloat16>, grid, smem_tw_fwd(a.d), st, a, sketch, lse_tok, stat_part);
   return run(&tw_fwd_kernel<float>, grid, smem_tw_fwd(a.d), st, a, sketch, lse_tok, stat_part);
-}
-
-cudaError_t launch_tw_finalize(const Args& a, int W, const float2* stat_part, float* sketch, float* lse_tok,
-                               cudaStream_t st) {
-  tw_finalize_kernel<<<a.B * a.H, 256, 0, st>>>(a.ws, a.prefix, a.B, a.H, a.P, a.d, W, a.partial, stat_part,
-                                                sketch, lse_tok);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_tw_dcoef(const Args& a, const float* O, const float* G, bool round_g, float* D,
