@@ -171,6 +171,7 @@ sa::Args make_args(const void* K, const void* V, const int32_t* cu, int B, int64
   a.lse_part = reinterpret_cast<float2*>(base + L.lse_part);
   a.uq = 0;
   a.dq_user = nullptr;
+  a.sum_dx = 0;
   return a;
 }
 
@@ -309,9 +310,10 @@ sa_status fwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
 
 // Backward of both entry points; uq = 1: Q and dQ hold one [H, P, d] block per
 // user, whose pieces from different workers are summed like the sketch's.
+// sum_dx = 1 (shapes with bwd_on_tc): dV receives dV + dK and dK is not written.
 sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int B, int64_t N, const void* Q, int H,
                    int P, int d, float scale, sa_dtype dt, const float* dsketch, const float* lse, void* dK,
-                   void* dV, float* dQ, void* workspace, size_t ws_bytes, void* stream, int uq) {
+                   void* dV, float* dQ, void* workspace, size_t ws_bytes, void* stream, int uq, int sum_dx = 0) {
   if (!dsketch || !dQ || (N > 0 && (!dK || !dV))) return SA_ERR_INVALID_ARG;
   Plan plan;
   SA_TRY(check_common(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, ws_bytes, true, uq, &plan));
@@ -319,6 +321,7 @@ sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
   sa::Args a = make_args(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, plan.lay);
   a.uq = uq;
   a.dq_user = uq ? dQ : nullptr;
+  a.sum_dx = sum_dx;
   const bool folded = plan.bwd_path == Path::TcBwd && scale < 0.f;
   // dQ from the per-worker pieces: summed over workers per head (shared
   // queries) or, per user, only for segments cut across workers
@@ -399,10 +402,14 @@ sa_status sa_sketch_bwd_per_user(const void* K, const void* V, const int32_t* cu
 static size_t x_elem(sa_dtype dt) { return dt == SA_BF16 ? 2 : 4; }
 
 // Extra workspace of the X entry points, after the step's own: Q' = Q W_K^T
-// [H,P,d] (dt); for the backward also dK' [N,H,d] (dt) and dQ' [H,P,d] (fp32).
+// [H,P,d] (dt); for the backward also dQ' [H,P,d] (fp32) and, on the CUDA cores,
+// dK' [N,H,d] (dt), which the tensor-core backward adds to dV in its epilogue.
+static bool x_sums_dx(int P, int d, sa_dtype dt) { return sa::tc_bwd_supported(P, d, dt); }
+
 static size_t x_extra(int64_t N, int H, int P, int d, sa_dtype dt, bool bwd) {
   size_t b = sa::align256(size_t(H) * P * d * x_elem(dt));
-  if (bwd) b += sa::align256(size_t(N) * H * d * x_elem(dt)) + sa::align256(size_t(H) * P * d * 4);
+  if (bwd) b += sa::align256(size_t(H) * P * d * 4);
+  if (bwd && !x_sums_dx(P, d, dt)) b += sa::align256(size_t(N) * H * d * x_elem(dt));
   return b;
 }
 
@@ -436,13 +443,16 @@ sa_status sa_sketch_bwd_x(const void* X, const int32_t* cu_seqlens, int B, int64
   if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0 || !aligned16(Wk)) return SA_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* Qf = static_cast<char*>(workspace) + base;
-  char* dKf = Qf + sa::align256(size_t(H) * P * d * x_elem(dt));
-  float* dQf = reinterpret_cast<float*>(dKf + sa::align256(size_t(N) * H * d * x_elem(dt)));
+  float* dQf = reinterpret_cast<float*>(Qf + sa::align256(size_t(H) * P * d * x_elem(dt)));
+  char* dKf = reinterpret_cast<char*>(dQf) + sa::align256(size_t(H) * P * d * 4);
+  const bool sum_dx = x_sums_dx(P, d, dt);
   SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_fold_wk(Q, Wk, H, P, d, dt, Qf, st); }));
-  // the step with K = V = X and prototypes Q': dK' to the workspace, dV into dX
-  SA_TRY(bwd_impl(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, dsketch, lse, N > 0 ? dKf : nullptr, dX, dQf,
-                  workspace, base, stream, 0));
-  SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_add_into(dX, dKf, N * H * int64_t(d), dt, st); }));
+  // the step with K = V = X and prototypes Q': dX = dV + dK' from the backward's
+  // epilogue, or dV into dX and dK' to the workspace and a pass that adds them
+  SA_TRY(bwd_impl(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, dsketch, lse,
+                  N > 0 ? (sum_dx ? dX : dKf) : nullptr, dX, dQf, workspace, base, stream, 0, sum_dx ? 1 : 0));
+  if (!sum_dx)
+    SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_add_into(dX, dKf, N * H * int64_t(d), dt, st); }));
   return launch(SA_KERNEL_AUX, st, [&] { return sa::launch_wk_grads(dQf, Q, Wk, H, P, d, dt, dQ, dWk, st); });
 }
 

@@ -23,6 +23,7 @@ struct Args {
   float2* lse_part;    // [N][H][slices] per-slice (max, sum) of the lse pass when P >= 1024
   int uq;              // 1: per-user queries Q[B][H][P][d] and dQ[B][H][P][d] (stacked refinement)
   float* dq_user;      // per-user queries: the caller's dQ[B][H][P][d] (whole segments go there)
+  int sum_dx;          // 1 (tensor-core backward with K = V = X): dV's buffer takes dV + dK, dK's is not written
 };
 
 // Row of Q ([H or B*H][P][d]) that user b, head h reads.

@@ -85,10 +85,33 @@ __device__ __forceinline__ void store_row_bf16(uint32_t taddr, __nv_bfloat16* ds
   }
 }
 
+// the same for mul * (row at ta) + (row at tb), summed in fp32 and rounded once
+template <int NCOL>
+__device__ __forceinline__ void store_row_sum_bf16(uint32_t ta, uint32_t tb, __nv_bfloat16* dst, float mul,
+                                                   bool valid) {
+  float v[16], w[16];
+#pragma unroll
+  for (int c = 0; c < NCOL; c += 16) {
+    tmem_ld16(ta + c, v);
+    tmem_ld16(tb + c, w);
+    tmem_ld_wait();
+    if (valid) {
+      uint4* o = reinterpret_cast<uint4*>(dst + c);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = fmaf(v[k], mul, w[k]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        o[k] = make_uint4(pack_bf16(v[8 * k], v[8 * k + 1]), pack_bf16(v[8 * k + 2], v[8 * k + 3]),
+                          pack_bf16(v[8 * k + 4], v[8 * k + 5]), pack_bf16(v[8 * k + 6], v[8 * k + 7]));
+    }
+  }
+}
+
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-template <int D, int PS, int MODE>
+// SUM: K = V = X, and dV's buffer takes dV + dK (Args::sum_dx)
+template <int D, int PS, int MODE, bool SUM>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_bwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   const __grid_constant__ CUtensorMap tmQ, Args a, const float* __restrict__ dsk,
@@ -403,8 +426,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       // dK of the previous tile and, at the end of a head piece, dQ
       auto finish_prev = [&](const TileWalker& pw, bool last_of_hp) {
         if (MODE == kFull) {
-          __nv_bfloat16* dst = dK + ((pw.tok0 + row) * a.H + pw.h) * int64_t(D) + sw * (D / 2);
-          store_row_bf16<D / 2>(tmem + lane_off + C::DK_COL + sw * (D / 2), dst, a.scale, row < pw.n);
+          // the sum dV + dK reads dV's columns here: the next tile's dV is issued only
+          // after every warp has stored that tile's weights, which follow this
+          __nv_bfloat16* dst = (SUM ? dV : dK) + ((pw.tok0 + row) * a.H + pw.h) * int64_t(D) + sw * (D / 2);
+          if (SUM)
+            store_row_sum_bf16<D / 2>(tmem + lane_off + C::DK_COL + sw * (D / 2),
+                                      tmem + lane_off + C::DV_COL + sw * (D / 2), dst, a.scale, row < pw.n);
+          else
+            store_row_bf16<D / 2>(tmem + lane_off + C::DK_COL + sw * (D / 2), dst, a.scale, row < pw.n);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(dk_empty);
@@ -511,7 +540,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           // dV rows of this tile
           __nv_bfloat16* dst = dV + (tok * a.H + cur.h) * int64_t(D) + sw * (D / 2);
-          store_row_bf16<D / 2>(tmem + lane_off + C::DV_COL + sw * (D / 2), dst, 1.f, valid);
+          if (!SUM)
+            store_row_bf16<D / 2>(tmem + lane_off + C::DV_COL + sw * (D / 2), dst, 1.f, valid);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) {
@@ -582,7 +612,7 @@ static cudaError_t launch_bwd_t(const Args& a, int W, const float* dsk, const fl
   if (!make_kv_map(&tk, a.K, a.N, a.H, D) || !make_kv_map(&tv, a.V, a.N, a.H, D) ||
       !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, PS))
     return cudaErrorInvalidValue;
-  auto fn = &tc_bwd_kernel<D, PS, MODE>;
+  auto fn = a.sum_dx ? &tc_bwd_kernel<D, PS, MODE, true> : &tc_bwd_kernel<D, PS, MODE, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   dim3 grid(W, a.P / PS);
@@ -684,7 +714,8 @@ __device__ __forceinline__ int tok_qg_pair(int, int c) { return 1 + (c & 1); }
 // (Dco written here).  TW = true: token-wise weights (Sec. 5.1), lse and Dco
 // per prototype [B][H][P] (both read), so dS = A o (dA - D_j) goes to shared
 // memory in place of E and dK = scale dS Q needs no qbar.
-template <int D, int P, bool TW>
+// SUM: K = V = X, and dV's buffer takes dV + dK (Args::sum_dx; not token-wise).
+template <int D, int P, bool TW, bool SUM>
 __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmQ,
                                              const CUtensorMap& tmG, const CUtensorMap& tmDK,
                                              const CUtensorMap& tmDV, const Args& a, const float* __restrict__ lse,
@@ -1084,37 +1115,47 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
                            pack_bf16(x[8 * k + 4], x[8 * k + 5]), pack_bf16(x[8 * k + 6], x[8 * k + 7]));
           }
         };
+        // with K = V = X (SUM) one tile dV + dK, summed in fp32, goes to dV's buffer
         if (whole) {
           float x[32];
+          if (!SUM) {
 #pragma unroll
-          for (int cc = 0; cc < D / 2; cc += 32) {
-            tmem_ld32(tmem + lane_off + C::DV_COL + sw * (D / 2) + cc, x);
-            tmem_ld_wait();
-            put_half(x, cc);
+            for (int cc = 0; cc < D / 2; cc += 32) {
+              tmem_ld32(tmem + lane_off + C::DV_COL + sw * (D / 2) + cc, x);
+              tmem_ld_wait();
+              put_half(x, cc);
+            }
+            ok = stage_and_store(&tmDV, cur);
+            if (!ok) break;
           }
-          ok = stage_and_store(&tmDV, cur);
-          if (!ok) break;
           float uu[32], qb[32];
 #pragma unroll
           for (int cc = 0; cc < D / 2; cc += 32) {
             tmem_ld32(tmem + lane_off + C::U_COL + sw * (D / 2) + cc, uu);
             if (!TW) tmem_ld32(tmem + lane_off + C::QB_COL + sw * (D / 2) + cc, qb);
+            if (SUM) tmem_ld32(tmem + lane_off + C::DV_COL + sw * (D / 2) + cc, x);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) uu[j] = TW ? a.scale * uu[j] : a.scale * fmaf(-Dv, qb[j], uu[j]);
+            for (int j = 0; j < 32; ++j) {
+              uu[j] = TW ? a.scale * uu[j] : a.scale * fmaf(-Dv, qb[j], uu[j]);
+              if (SUM) uu[j] += x[j];
+            }
             put_half(uu, cc);
           }
-          ok = stage_and_store(&tmDK, cur);
+          ok = stage_and_store(SUM ? &tmDV : &tmDK, cur);
           if (!ok) break;
         } else {
           __nv_bfloat16* dvr = dV + (tok * a.H + cur.h) * int64_t(D) + sw * (D / 2);
-          store_row_bf16<D / 2>(tmem + lane_off + C::DV_COL + sw * (D / 2), dvr, 1.f, valid);
-          __nv_bfloat16* dkr = dK + (tok * a.H + cur.h) * int64_t(D) + sw * (D / 2);
+          if (!SUM) store_row_bf16<D / 2>(tmem + lane_off + C::DV_COL + sw * (D / 2), dvr, 1.f, valid);
+          __nv_bfloat16* dkr =
+              SUM ? dvr : dK + (tok * a.H + cur.h) * int64_t(D) + sw * (D / 2);
           float uu[32], qb[32];
 #pragma unroll
           for (int cc = 0; cc < D / 2; cc += 32) {
             tmem_ld32(tmem + lane_off + C::U_COL + sw * (D / 2) + cc, uu);
             if (!TW) tmem_ld32(tmem + lane_off + C::QB_COL + sw * (D / 2) + cc, qb);
+            float dv[32];
+            if (SUM) tmem_ld32(tmem + lane_off + C::DV_COL + sw * (D / 2) + cc, dv);
             tmem_ld_wait();
             if (valid) {
               uint4* o = reinterpret_cast<uint4*>(dkr + cc);
@@ -1122,8 +1163,10 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
               for (int k = 0; k < 4; ++k) {
                 float x[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < 8; ++j) {
                   x[j] = TW ? a.scale * uu[8 * k + j] : a.scale * fmaf(-Dv, qb[8 * k + j], uu[8 * k + j]);
+                  if (SUM) x[j] += dv[8 * k + j];
+                }
                 o[k] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]),
                                   pack_bf16(x[6], x[7]));
               }
@@ -1145,14 +1188,14 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
   }
 }
 
-template <int D, int P>
+template <int D, int P, bool SUM>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_bwd_tok_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
                       const __grid_constant__ CUtensorMap tmDK, const __grid_constant__ CUtensorMap tmDV, Args a,
                       const float* __restrict__ lse, float* __restrict__ Dco, __nv_bfloat16* __restrict__ dK,
                       __nv_bfloat16* __restrict__ dV) {
-  bwd_tok_body<D, P, false>(tmK, tmV, tmQ, tmG, tmDK, tmDV, a, lse, Dco, dK, dV);
+  bwd_tok_body<D, P, false, SUM>(tmK, tmV, tmQ, tmG, tmDK, tmDV, a, lse, Dco, dK, dV);
 }
 
 template <int D, int P>
@@ -1162,7 +1205,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                          const __grid_constant__ CUtensorMap tmDK, const __grid_constant__ CUtensorMap tmDV, Args a,
                          const float* __restrict__ lse_tok, float* __restrict__ Dtw, __nv_bfloat16* __restrict__ dK,
                          __nv_bfloat16* __restrict__ dV) {
-  bwd_tok_body<D, P, true>(tmK, tmV, tmQ, tmG, tmDK, tmDV, a, lse_tok, Dtw, dK, dV);
+  bwd_tok_body<D, P, true, false>(tmK, tmV, tmQ, tmG, tmDK, tmDV, a, lse_tok, Dtw, dK, dV);
 }
 
 // dsketch fp32 -> bf16 copy in the workspace, the layout TMA streams ([B*H][P][D])
@@ -1186,7 +1229,8 @@ static cudaError_t launch_tok_t(const Args& a, int W, const __nv_bfloat16* gbf, 
       !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, C::NC) || !make_q_map(&tg, gbf, a.B * a.H, a.P, D, C::NC) ||
       !make_kv_map(&tdk, dK, a.N, a.H, D) || !make_kv_map(&tdv, dV, a.N, a.H, D))
     return cudaErrorInvalidValue;
-  auto fn = TW ? &tc_tw_bwd_tok_kernel<D, P> : &tc_bwd_tok_kernel<D, P>;
+  auto fn = &tc_tw_bwd_tok_kernel<D, P>;
+  if constexpr (!TW) fn = a.sum_dx ? &tc_bwd_tok_kernel<D, P, true> : &tc_bwd_tok_kernel<D, P, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   fn<<<W, kThreads, C::SMEM, st>>>(tk, tv, tq, tg, tdk, tdv, a, lse, Dco, static_cast<__nv_bfloat16*>(dK),
