@@ -1,6 +1,5 @@
 // Staging helpers of the CUDA-core kernels (sa_simt.cu, sa_tokenwise.cu):
-// vector loads widened to fp32, rows copied into padded shared-memory tiles,
-// and the user that holds a token.
+// vector loads widened to fp32 and rows copied into padded shared-memory tiles.
 #pragma once
 #include "sa_kernels.cuh"
 
@@ -54,17 +53,6 @@ __device__ __forceinline__ void stage_rows_f32(float* dst, const float* src, int
     const int r = e / d, c = e - r * d;
     dst[r * (d + 1) + c] = r < nrows ? src[int64_t(r) * d + c] : 0.f;
   }
-}
-
-// User of token t: the largest b with cu[b] <= t (empty users before it share
-// its offset, so the largest such b is the user that holds t).
-__device__ __forceinline__ int user_of_token(const int32_t* cu, int B, int64_t t) {
-  int lo = 0, hi = B - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (int64_t(cu[mid]) <= t) lo = mid; else hi = mid - 1;
-  }
-  return lo;
 }
 
 }  // namespace sa
