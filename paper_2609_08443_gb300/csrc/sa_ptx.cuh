@@ -100,6 +100,33 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, ws, site));
 }
 
+// Several barriers at once.  A shared-memory access takes 250-400 cycles beside
+// running tensor-core products, so the polls are issued back to back and their
+// latencies overlap; only what is not complete yet is then waited for in turn.
+struct BarPhase {
+  uint32_t bar, parity;
+};
+template <int N>
+__device__ __forceinline__ bool mbar_wait_warp_all(const BarPhase (&b)[N], volatile int* abort_flag, void* ws,
+                                                   uint32_t site) {
+  bool done[N], all = true;
+#pragma unroll
+  for (int k = 0; k < N; ++k) done[k] = mbar_try_wait(b[k].bar, b[k].parity);
+#pragma unroll
+  for (int k = 0; k < N; ++k) all = all && done[k];
+  if (__all_sync(0xffffffffu, all)) return true;
+  bool ok = true;
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) {
+    uint32_t bar = b[0].bar, parity = b[0].parity;
+#pragma unroll
+    for (int j = 1; j < N; ++j)
+      if (k == j) bar = b[j].bar, parity = b[j].parity;
+    ok = ok && mbar_wait(bar, parity, abort_flag, ws, site);
+  }
+  return __all_sync(0xffffffffu, ok);
+}
+
 // True in one lane of a converged warp (always the same lane).  The UMMA
 // issuers run as whole warps and issue under this predicate: the compiler then
 // knows that one thread executes the block and keeps descriptors in uniform
@@ -197,6 +224,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint
       " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
+}
+
+// Contiguous copy, global -> shared: both addresses and the size are multiples of 16.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
+               : "memory");
 }
 
 // Pull a tile into L2 ahead of its shared-memory load (no completion tracking).

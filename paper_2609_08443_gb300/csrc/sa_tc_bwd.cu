@@ -710,8 +710,8 @@ __host__ __device__ constexpr int tok_da_col() {
 __device__ __forceinline__ int tok_kv_pair(int) { return 0; }
 __device__ __forceinline__ int tok_qg_pair(int, int c) { return 1 + (c & 1); }
 
-// TW = false: prototype-wise weights (Sec. 3.1), lse and Dco per token [N][H]
-// (Dco written here).  TW = true: token-wise weights (Sec. 5.1), lse and Dco
+// TW = false: prototype-wise weights (Sec. 3.1), lse per token [N][H]; Dco is
+// written here, float2 [H][N] (lse log2 e, D_i).  TW = true: token-wise weights (Sec. 5.1), lse and Dco
 // per prototype [B][H][P] (both read), so dS = A o (dA - D_j) goes to shared
 // memory in place of E and dK = scale dS Q needs no qbar.
 // SUM: K = V = X, and dV's buffer takes dV + dK (Args::sum_dx; not token-wise).
@@ -1097,7 +1097,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
           Dv = stats[row] + stats[T + row];
           __syncwarp();
           if (lane == 0) mbar_arrive(st_used);
-          if (sw == 0 && valid) Dco[tok * a.H + cur.h] = Dv;
+          if (sw == 0 && valid) reinterpret_cast<float2*>(Dco)[int64_t(cur.h) * a.N + tok] = make_float2(L2, Dv);
         }
         // epilogue: dV and dK = scale (u - D qbar); this warpgroup owns columns [sw*D/2, +D/2)
         ok = wwait(acc_full, li & 1, 0xA07);
@@ -1266,9 +1266,6 @@ cudaError_t launch_tc_bwd_tok(const Args& a, int W, const float* dsk, __nv_bfloa
   return tcb::launch_tok_t<128, 256>(a, W, gbf, lse, Dco, dK, dV, st);
 }
 
-cudaError_t launch_tc_bwd_dq(const Args& a, int W, const float* dsk, const float* lse, const float* Dco,
-                             cudaStream_t st);
-
 int tc_bwd_dq_workers(int num_sms, int P) {
   const int w = num_sms / (P / 128);
   return w < 1 ? 1 : w;
@@ -1276,469 +1273,7 @@ int tc_bwd_dq_workers(int num_sms, int P) {
 
 }  // namespace sa
 
-// ================================================================ dQ (slices)
-// Prototype side of the backward: one slice of PS = 128 prototypes per CTA,
-// prototypes on TMEM lanes, tokens on columns:
-//   S  = Q_r K^T,  dA = G_r V^T                (UMMA, [PS x 128 tokens])
-//   dS = exp(scale S - lse_t) o (dA - D_t)     (registers; lse_t and D_t are
-//                                               per-column values, no reduction)
-//   dQ_r += dS K                               (UMMA with dS as the A operand
-//                                               straight from TMEM)
-// D_t comes from the token-side kernel.  Keeping dS in TMEM spares the
-// shared-memory round trip that bounds the other kernels.
 namespace sa {
-namespace tcb {
-
-template <int D, int PS>
-struct QCfg {
-  static constexpr int KV_TILE = T * D * 2;
-  static constexpr int QB = PS * D * 2;
-  // K(i) is read by S(i) and, a tile later, by dQ(i); V(i) only by dA(i).  So
-  // K gets four slots and V two: K(i+3) loads once dQ(i-1) is done and V(i+2)
-  // once dA(i) is, a tile or more before they are needed.  (The dsketch slice
-  // lives in TMEM as the A operand of dA, which leaves room for the fourth.)
-  static constexpr int NK = 4, NV = 2;
-  static constexpr int NSLOT = NK + NV;
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_RING = QB;  // K slots 0..NK-1, then V slots
-  static constexpr int OFF_COL = OFF_RING + NSLOT * KV_TILE;  // [2 bufs][lse2 | D][128] fp32
-  static constexpr int OFF_BAR = OFF_COL + 2 * 2 * T * 4;
-  static constexpr int NBAR = 2 * NSLOT + 16;
-  static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;  // TMEM base, abort flag
-  static constexpr int OFF_FLAGS = OFF_MISC + 16;      // per K slot: control bits of the tile it holds
-  static constexpr int SMEM = OFF_FLAGS + 4 * NK;
-  // S^T and dA^T fp32; dS (bf16 pairs) and the dsketch slice G (bf16 pairs, the
-  // A operand of dA^T = G V^T) 64 columns each; dQ fp32
-  static constexpr int S_COL = 0, DA_COL = T, DS_COL = 2 * T, G_COL = 2 * T + T / 2, DQ_COL = 3 * T;
-  static constexpr int TMEM_COLS = tmem_cols_for(DQ_COL + D);
-  static_assert(PS == 128 && TMEM_COLS <= 512 && SMEM <= 232448, "budget");
-};
-
-// Per-tile control bits, written by the TMA producer next to the tile's K so
-// the UMMA issuer follows the tile sequence without walking it.
-enum : uint32_t { kNewHead = 1u, kHeadLast = 2u, kSegFirst = 4u, kSegLast = 8u };
-
-// TW = false: prototype-wise weights, lse and D per token (column values
-// staged by warps 2-3).  TW = true: token-wise weights (Sec. 5.1), lse and D
-// per prototype [B][H][P]: per-row (per-thread) values, and columns past the
-// tile's tokens are masked here.
-template <int D, int PS, bool TW>
-__device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmQ,
-                                            const Args& a, const float* __restrict__ dsk,
-                                            const float* __restrict__ lse, const float* __restrict__ Dco) {
-  using C = QCfg<D, PS>;
-  extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  if (ws_failed(a.ws)) return;
-  if (smem_u32(smem) & 1023u) {
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB31u);
-    return;
-  }
-  const uint32_t sbase = smem_u32(smem);
-  const uint32_t sQ = sbase + C::OFF_Q, sRing = sbase + C::OFF_RING;
-  const uint32_t bar0 = sbase + C::OFF_BAR;
-  // slot s < NK holds K tiles, slot NK + j holds V tiles
-  auto ring_full = [&](int s) { return bar0 + 8u * s; };
-  auto ring_empty = [&](int s) { return bar0 + 8u * (C::NSLOT + s); };
-  auto k_slot = [](int li) { return li % C::NK; };
-  auto v_slot = [](int li) { return C::NK + li % C::NV; };
-  const uint32_t b1 = bar0 + 8u * (2 * C::NSLOT);
-  const uint32_t q_full = b1, q_empty = b1 + 8, g_full = b1 + 16, g_empty = b1 + 24, sda_full = b1 + 32,
-                 sda_free = b1 + 40, ds_full = b1 + 48, ds_empty0 = b1 + 56, dq_empty = b1 + 72,
-                 col_full0 = b1 + 80, col_empty0 = b1 + 96, drain = b1 + 112;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
-  uint32_t* tflags = reinterpret_cast<uint32_t*>(smem + C::OFF_FLAGS);
-  float* cols = reinterpret_cast<float*>(smem + C::OFF_COL);
-  const int64_t tph = reinterpret_cast<const WsHeader*>(a.ws)->tiles_per_head;
-  const int64_t total = tph * a.H;
-  const int W = gridDim.x, wk = blockIdx.x, slice = blockIdx.y;
-  const int p0 = slice * PS;
-  const int64_t tb = range_begin(total, W, wk), te = range_begin(total, W, wk + 1);
-  const int ntiles = int(te - tb);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < C::NSLOT; ++s) {
-      mbar_init(ring_full(s), 1);
-      mbar_init(ring_empty(s), 1);
-    }
-    mbar_init(q_full, 1);
-    mbar_init(q_empty, 1);
-    mbar_init(g_full, kSoftWarps);
-    mbar_init(g_empty, 1);
-    mbar_init(sda_full, 1);
-    mbar_init(sda_free, kSoftWarps);
-    mbar_init(ds_full, kSoftWarps);
-    mbar_init(ds_empty0, 1);
-    mbar_init(ds_empty0 + 8, 1);  // unused (one dS buffer)
-    mbar_init(dq_empty, kSoftWarps);
-    mbar_init(col_full0, 2);
-    mbar_init(col_full0 + 8, 2);
-    mbar_init(col_empty0, kSoftWarps);
-    mbar_init(col_empty0 + 8, kSoftWarps);
-    mbar_init(drain, 1);
-    wait_ctl_init(abort_flag, a.ws);
-    fence_mbar_init();
-  }
-  if (warp == 2) tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-
-  // Registers: the control warpgroup (warps 0-3: TMA, UMMA issuer, column loaders)
-  // hands registers to the two softmax warpgroups (128 x 136 + 256 x 184 = 384 x 168).
-  if (ntiles > 0 && warp < kSoftWarp0) {
-    setmaxnreg_dec<136>();
-    if (warp == 0 && lane == 0) {
-      // ---------------------------------------------------------- TMA producer
-      tma_prefetch_desc(&tmK);
-      tma_prefetch_desc(&tmV);
-      tma_prefetch_desc(&tmQ);
-      TileWalker it(a, tb, te, T);
-      int hc = 0, prev_h = -1, loaded = 0;
-      bool ok = true;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        // "head" below = the run of tiles reading one row of Q: a head, or with
-        // per-user queries one (user, head) segment
-        const bool new_head = it.qk != prev_h;
-        if (new_head) {
-          if (hc > 0) ok = mbar_wait(q_empty, (hc - 1) & 1, abort_flag, a.ws, 0xC01);
-          if (!ok) break;
-          mbar_arrive_expect_tx(q_full, C::QB);
-#pragma unroll
-          for (int dh = 0; dh < D / 64; ++dh) tma_load_3d(sQ + dh * PS * 128, &tmQ, q_full, 64 * dh, p0, it.qk);
-          prev_h = it.qk;
-          ++hc;
-        }
-        int64_t t0n;
-        int nn, hn, qkn;
-        it.peek_next(t0n, nn, hn, qkn);
-        const uint32_t fl = (new_head ? kNewHead : 0u) | ((li + 1 >= ntiles || qkn != it.qk) ? kHeadLast : 0u) |
-                            (it.seg_first ? kSegFirst : 0u) | (it.seg_last ? kSegLast : 0u);
-#pragma unroll
-        for (int kv = 0; kv < 2; ++kv) {
-          const int nsl = kv ? C::NV : C::NK, use = li / nsl;
-          const int s = kv ? v_slot(li) : k_slot(li);
-          if (use > 0) ok = mbar_wait(ring_empty(s), (use + 1) & 1, abort_flag, a.ws, 0xC02);
-          if (!ok) break;
-          if (kv == 0) tflags[s] = fl;  // published by the arrive below
-          mbar_arrive_expect_tx(ring_full(s), C::KV_TILE);
-#pragma unroll
-          for (int dh = 0; dh < D / 64; ++dh)
-            tma_load_3d(sRing + s * C::KV_TILE + dh * T * 128, kv ? &tmV : &tmK, ring_full(s), 64 * dh, it.h,
-                        int(it.tok0));
-          loaded = li + 1;
-        }
-        it.next();
-      }
-      if (!ok) {  // let the copies in flight land before the CTA exits
-        for (int li = (loaded > C::NK ? loaded - C::NK : 0); li < loaded; ++li) {
-          mbar_wait_bounded(ring_full(k_slot(li)), (li / C::NK) & 1, 200000000ull);
-          if (li + C::NV >= loaded) mbar_wait_bounded(ring_full(v_slot(li)), (li / C::NV) & 1, 200000000ull);
-        }
-      }
-    } else if (warp == 1) {
-      // ---------------------------------------------------------- UMMA issuer
-      // Order: S(0), dA(0);
-      // then per tile i: S(i+1), dA(i+1), dQ(i), so the next tile's scores are
-      // ready when the softmax warps finish tile i.  One commit announces S and
-      // dA together (the softmax warps read both at once); descriptors are
-      // built once per operand and stepped by constant offsets.
-      constexpr uint32_t idPT = idesc_bf16(128, T, 0, 0);  // [proto x tok], K = d
-      constexpr uint32_t idQ = idesc_bf16(128, D, 0, 1);   // [proto x d], K = tokens, A from TMEM
-      const uint64_t dQs = sdesc(sQ, 16, 1024);
-      auto step_p = [](int k) { return uint32_t((k >> 2) * (PS * 128) + (k & 3) * 32); };
-      auto step_t = [](int k) { return uint32_t((k >> 2) * (T * 128) + (k & 3) * 32); };
-      int hc = 0, gc = 0, hp = 0;
-      bool ok = true;
-      auto wt = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return ok = ok && mbar_wait_warp(bar, par, abort_flag, a.ws, site);
-      };
-      // waits for tile li's K and V, returns its control bits
-      auto wait_kv = [&](int li) -> uint32_t {
-        wt(ring_full(k_slot(li)), (li / C::NK) & 1, 0xD02);
-        wt(ring_full(v_slot(li)), (li / C::NV) & 1, 0xD04);
-        return ok ? tflags[k_slot(li)] : 0u;
-      };
-      auto issue_sda = [&](int li, uint32_t fl) {
-        if (fl & kNewHead) {
-          wt(q_full, hc & 1, 0xD01);
-          ++hc;
-        }
-        if (fl & kSegFirst) {
-          wt(g_full, gc & 1, 0xD03);
-          ++gc;
-        }
-        if (!ok) return;
-        tc_fence_after();
-        const int sK = k_slot(li), sV = v_slot(li);
-        const uint64_t dK = sdesc(sRing + sK * C::KV_TILE, 16, 1024), dV = sdesc(sRing + sV * C::KV_TILE, 16, 1024);
-        if (elect_one()) {
-#pragma unroll
-          for (int k = 0; k < D / 16; ++k)
-            umma_ss(tmem + C::S_COL, sdesc_add(dQs, step_p(k)), sdesc_add(dK, step_t(k)), idPT, k > 0 ? 1u : 0u);
-#pragma unroll
-          for (int k = 0; k < D / 16; ++k)  // G from TMEM: 8 columns (16 values of d) per step
-            umma_ts(tmem + C::DA_COL, tmem + C::G_COL + 8 * k, sdesc_add(dV, step_t(k)), idPT, k > 0 ? 1u : 0u);
-          umma_commit(sda_full);
-          umma_commit(ring_empty(sV));                // V read by its only product
-          if (fl & kHeadLast) umma_commit(q_empty);   // last S of this head piece
-          if (fl & kSegLast) umma_commit(g_empty);    // last dA of this segment
-        }
-      };
-      uint32_t fl_cur = wait_kv(0);
-      if (ok) issue_sda(0, fl_cur);
-      for (int li = 0; li < ntiles && ok; ++li) {
-        uint32_t fl_next = 0;
-        if (li + 1 < ntiles) {
-          wt(sda_free, li & 1, 0xD07);  // the softmax warps hold S(i), dA(i)
-          fl_next = wait_kv(li + 1);
-          if (!ok) break;
-          issue_sda(li + 1, fl_next);
-          if (!ok) break;
-        }
-        // ---- dQ += dS(i) K(i), dS read from TMEM
-        const bool first_of_hp = (fl_cur & kNewHead) != 0;
-        wt(ds_full, li & 1, 0xD09);
-        if (first_of_hp && hp > 0) wt(dq_empty, (hp - 1) & 1, 0xD0A);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
-          const int sK = k_slot(li);
-          const uint64_t dK = sdesc(sRing + sK * C::KV_TILE, T * 128, 1024);  // MN-major: d blocks 16 KB apart
-          const uint32_t dsb = tmem + C::DS_COL;
-#pragma unroll
-          for (int k = 0; k < T / 16; ++k)
-            umma_ts(tmem + C::DQ_COL, dsb + 8 * k, sdesc_add(dK, k * 2048), idQ, (first_of_hp && k == 0) ? 0u : 1u);
-          umma_commit(ds_empty0);
-          umma_commit(ring_empty(sK));
-        }
-        if (fl_cur & kHeadLast) ++hp;
-        fl_cur = fl_next;
-      }
-      if (elect_one()) umma_commit(drain);
-      mbar_wait_bounded(drain, 0, 200000000ull);
-    } else if (warp == 2 || warp == 3) {
-      // ------------------------------------------------- per-token columns
-      const int t64 = threadIdx.x - 64;
-      TileWalker cur(a, tb, te, T);
-      bool ok = true;
-      auto hw = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return __all_sync(0xffffffffu, mbar_wait(bar, par, abort_flag, a.ws, site));
-      };
-      for (int li = 0; li < ntiles && ok; ++li) {
-        if (!TW) {
-          const int buf = li & 1;
-          if (li >= 2) ok = hw(col_empty0 + 8 * buf, ((li >> 1) + 1) & 1, 0xE02);
-          if (!ok) break;
-          float* cl = cols + buf * 2 * T;
-          for (int t = t64; t < T; t += 64) {
-            const bool v = t < cur.n;
-            const int64_t idx = (cur.tok0 + t) * a.H + cur.h;
-            cl[t] = v ? lse[idx] * 1.4426950408889634f : INFINITY;  // exp2(x - inf) = 0 for padding
-            cl[T + t] = v ? Dco[idx] : 0.f;
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(col_full0 + 8 * buf);
-        }
-        cur.next();
-      }
-    }
-  } else if (ntiles > 0) {
-    setmaxnreg_inc<184>();
-    {
-      // ------------------------------------------------ dS + dQ epilogue
-      const int sw = (warp - kSoftWarp0) >> 2, q = warp & 3;
-      const uint32_t lane_off = uint32_t(32 * q) << 16;
-      const float c2 = a.scale * 1.4426950408889634f;
-      TileWalker cur(a, tb, te, T);
-      bool ok = true;
-      int gc = 0;
-      // The dsketch slice of user b, head h into TMEM as bf16 pairs (the A operand of
-      // dA^T = G V^T): this thread's prototype row, warpgroup sw's half of the d columns.
-      // Written once the last dA of the previous segment is done (g_empty).
-      auto put_g = [&](int b, int h) -> bool {
-        if (gc > 0 && !__all_sync(0xffffffffu, mbar_wait(g_empty, (gc - 1) & 1, abort_flag, a.ws, 0xF06)))
-          return false;
-        const float4* src = reinterpret_cast<const float4*>(
-            dsk + ((int64_t(b) * a.H + h) * a.P + p0 + 32 * q + lane) * D + (D / 2) * sw);
-#pragma unroll
-        for (int half = 0; half < D / 64; ++half) {
-          uint32_t pk[16];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 x = src[8 * half + j];
-            pk[2 * j] = pack_bf16(x.x, x.y);
-            pk[2 * j + 1] = pack_bf16(x.z, x.w);
-          }
-          tmem_st16(tmem + lane_off + C::G_COL + (D / 4) * sw + 16 * half, pk);
-        }
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(g_full);
-        ++gc;
-        return true;
-      };
-      ok = put_g(cur.b, cur.h);
-      auto wwait = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return __all_sync(0xffffffffu, mbar_wait(bar, par, abort_flag, a.ws, site));
-      };
-      int hp = 0;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        const int buf = li & 1;
-        float l2r = 0.f, dr = 0.f;  // token-wise: this row's lse (log2 units) and D
-        if (TW) {
-          const int64_t r = (int64_t(cur.b) * a.H + cur.h) * a.P + p0 + 32 * q + lane;
-          l2r = lse[r] * 1.4426950408889634f;
-          dr = Dco[r];
-        } else {
-          ok = wwait(col_full0 + 8 * buf, (li >> 1) & 1, 0xF01);
-        }
-        if (ok) ok = wwait(sda_full, li & 1, 0xF02);
-        if (!ok) break;
-        tc_fence_after();
-        const float* cl = cols + buf * 2 * T;
-        float sv[64], dv[64];  // this warpgroup's 64 token columns of S and dA
-        tmem_ld32(tmem + lane_off + C::S_COL + 64 * sw, sv);
-        tmem_ld32(tmem + lane_off + C::S_COL + 64 * sw + 32, sv + 32);
-        tmem_ld32(tmem + lane_off + C::DA_COL + 64 * sw, dv);
-        tmem_ld32(tmem + lane_off + C::DA_COL + 64 * sw + 32, dv + 32);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        // the next tile opens a new (user, head) segment: its dsketch slice goes in
-        // before S and dA of that tile are issued (they wait for sda_free and g_full)
-        if (li + 1 < ntiles && cur.seg_last) {
-          const TileRef nx = locate_next_segment(cur.t + 1, cur.h, cur.b, cur.tph, a.prefix, a.cu, a.B, T);
-          if (!put_g(nx.b, nx.h)) {
-            ok = false;
-            break;
-          }
-        }
-        if (lane == 0) mbar_arrive(sda_free);  // the next tile's S and dA may now be written
-        if (TW) {
-          // per-row shift and D; columns past the tile's tokens weigh zero
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int col = 64 * sw + 32 * c;
-            uint32_t pk[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int jj = 32 * c + 2 * j;
-              const float a0 = col + 2 * j < cur.n ? ex2(fmaf(sv[jj], c2, -l2r)) : 0.f;
-              const float a1 = col + 2 * j + 1 < cur.n ? ex2(fmaf(sv[jj + 1], c2, -l2r)) : 0.f;
-              pk[j] = pack_bf16(a0 * (dv[jj] - dr), a1 * (dv[jj + 1] - dr));
-            }
-            // dS(i) overwrites dS(i-1): dQ(i-1) must have read it
-            if (c == 0 && li > 0 && !wwait(ds_empty0, (li - 1) & 1, 0xF04)) {
-              ok = false;
-              break;
-            }
-            tmem_st16(tmem + lane_off + C::DS_COL + col / 2, pk);
-          }
-          if (!ok) break;
-        }
-        // per-token values as 16-byte broadcasts: one shared-memory wavefront per 4 tokens
-        const float4* cl4 = reinterpret_cast<const float4*>(cl);
-#pragma unroll
-        for (int c = 0; c < 2 && !TW; ++c) {
-          const int col = 64 * sw + 32 * c;
-          uint32_t pk[16];
-#pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4) {
-            const float4 l4 = cl4[(col >> 2) + j4];
-            const float4 d4 = cl4[((T + col) >> 2) + j4];
-            const int jj = 32 * c + 4 * j4;
-            const float a0 = ex2(fmaf(sv[jj], c2, -l4.x)), a1 = ex2(fmaf(sv[jj + 1], c2, -l4.y));
-            const float a2 = ex2(fmaf(sv[jj + 2], c2, -l4.z)), a3 = ex2(fmaf(sv[jj + 3], c2, -l4.w));
-            pk[2 * j4] = pack_bf16(a0 * (dv[jj] - d4.x), a1 * (dv[jj + 1] - d4.y));
-            pk[2 * j4 + 1] = pack_bf16(a2 * (dv[jj + 2] - d4.z), a3 * (dv[jj + 3] - d4.w));
-          }
-          if (c == 0 && li > 0 && !wwait(ds_empty0, (li - 1) & 1, 0xF04)) {
-            ok = false;
-            break;
-          }
-          tmem_st16(tmem + lane_off + C::DS_COL + col / 2, pk);
-        }
-        if (!ok) break;
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(ds_full);
-          if (!TW) mbar_arrive(col_empty0 + 8 * buf);
-        }
-        // dQ partial of this worker and head (or user segment) at the end of its piece
-        const bool more = li + 1 < ntiles;
-        int64_t t0n;
-        int nn, hn, qkn;
-        cur.peek_next(t0n, nn, hn, qkn);
-        if (!more || qkn != cur.qk) {
-          ok = wwait(ds_empty0, li & 1, 0xF05);
-          if (!ok) break;
-          tc_fence_after();
-          float* dst = dq_block_dst(a, wk, W, total, cur, p0, D);
-          store_sketch_scaled<D, PS, C::DQ_COL>(tmem, lane_off, sw, q, lane, dst, a.scale);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(dq_empty);
-          ++hp;
-        }
-        cur.next();
-      }
-      (void)hp;
-    }
-  }
-  __syncthreads();
-  if (warp == 2) {
-    tc_fence_after();
-    tmem_dealloc(tmem, C::TMEM_COLS);
-  }
-}
-
-template <int D, int PS>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                     const __grid_constant__ CUtensorMap tmQ, Args a, const float* __restrict__ dsk,
-                     const float* __restrict__ lse, const float* __restrict__ Dco) {
-  bwd_dq_body<D, PS, false>(tmK, tmV, tmQ, a, dsk, lse, Dco);
-}
-
-template <int D, int PS>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_tw_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                        const __grid_constant__ CUtensorMap tmQ, Args a, const float* __restrict__ dsk,
-                        const float* __restrict__ lse_tok, const float* __restrict__ Dtw) {
-  bwd_dq_body<D, PS, true>(tmK, tmV, tmQ, a, dsk, lse_tok, Dtw);
-}
-
-template <int D, int PS, bool TW = false>
-static cudaError_t launch_dq_t(const Args& a, int W, const float* dsk, const float* lse, const float* Dco,
-                               cudaStream_t st) {
-  using C = QCfg<D, PS>;
-  CUtensorMap tk, tv, tq;
-  if (!make_kv_map(&tk, a.K, a.N, a.H, D) || !make_kv_map(&tv, a.V, a.N, a.H, D) ||
-      !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, PS))
-    return cudaErrorInvalidValue;
-  auto fn = TW ? &tc_tw_bwd_dq_kernel<D, PS> : &tc_bwd_dq_kernel<D, PS>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-  if (e != cudaSuccess) return e;
-  dim3 grid(W, a.P / PS);
-  fn<<<grid, kThreads, C::SMEM, st>>>(tk, tv, tq, a, dsk, lse, Dco);
-  return cudaGetLastError();
-}
-
-}  // namespace tcb
-}  // namespace sa
-
-namespace sa {
-cudaError_t launch_tc_bwd_dq(const Args& a, int W, const float* dsk, const float* lse, const float* Dco,
-                             cudaStream_t st) {
-  if (a.N == 0) return cudaSuccess;
-  return a.d == 64 ? tcb::launch_dq_t<64, 128>(a, W, dsk, lse, Dco, st) : tcb::launch_dq_t<128, 128>(a, W, dsk, lse, Dco, st);
-}
-
 // Token-wise normalisation (Sec. 5.1): the same two kernels with per-prototype
 // lse_tok and D_j = G_j . O_j ([B][H][P]); d = 128 and P in {256, ..., 2048}.
 bool tc_tw_bwd_supported(int P, int d, sa_dtype dt) {
@@ -1756,9 +1291,4 @@ cudaError_t launch_tc_tw_bwd_tok(const Args& a, int W, const __nv_bfloat16* gbf,
   return tcb::launch_tok_t<128, 256, true>(a, W, gbf, lse_tok, Dp, dK, dV, st);
 }
 
-cudaError_t launch_tc_tw_bwd_dq(const Args& a, int W, const float* dsk, const float* lse_tok, const float* Dtw,
-                                cudaStream_t st) {
-  if (a.N == 0) return cudaSuccess;
-  return tcb::launch_dq_t<128, 128, true>(a, W, dsk, lse_tok, Dtw, st);
-}
 }  // namespace sa
