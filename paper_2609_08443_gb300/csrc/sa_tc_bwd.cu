@@ -273,8 +273,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           wt(g_full_of(gbuf), uint32_t(gc / C::NG) & 1u, 0x503);
           ++gc;
         }
-        wt(ring_full(sV), (eV / C::NSLOT) & 1, 0x504);
-        wt(sd_free_s, li & 1, 0x505);
+        {
+          const BarPhase both[2] = {{ring_full(sV), (eV / C::NSLOT) & 1}, {sd_free_s, uint32_t(li) & 1u}};
+          ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x504);
+        }
         if (!ok) break;
         tc_fence_after();
         const uint32_t gofs = uint32_t(gbuf * C::Q_BYTES);  // this segment's dsketch buffer
@@ -289,8 +291,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // ---- dV(i) = A G
         if (MODE == kFull) {
-          wt(a_full, li & 1, 0x506);
-          if (li > 0) wt(dv_empty, (li - 1) & 1, 0x507);
+          const BarPhase af{a_full, uint32_t(li) & 1u};
+          const BarPhase both[2] = {af, li > 0 ? BarPhase{dv_empty, uint32_t(li - 1) & 1u} : af};
+          ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x506);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -315,10 +318,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               wt(q_full, hc & 1, 0x508);
             }
             if (li >= 1) wt(sd_free_da, (li - 1) & 1, 0x509);
+            wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x50A);
           } else {
-            wt(sd_free_da, li & 1, 0x509);
+            const BarPhase both[2] = {{sd_free_da, uint32_t(li) & 1u},
+                                      {ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1}};
+            ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x509);
           }
-          wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x50A);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -328,9 +333,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         // ---- dK(i) = dS Q, dQ += dS^T K
-        wt(ds_full, li & 1, 0x50B);
-        if (MODE == kFull && li > 0) wt(dk_empty, (li - 1) & 1, 0x50C);
-        if (first_of_hp && hp > 0) wt(dq_empty, (hp - 1) & 1, 0x50D);
+        {
+          const BarPhase df{ds_full, uint32_t(li) & 1u};
+          const BarPhase three[3] = {df, MODE == kFull && li > 0 ? BarPhase{dk_empty, uint32_t(li - 1) & 1u} : df,
+                                     first_of_hp && hp > 0 ? BarPhase{dq_empty, uint32_t(hp - 1) & 1u} : df};
+          ok = ok && mbar_wait_warp_all(three, abort_flag, a.ws, 0x50B);
+        }
         if (!ok) break;
         tc_fence_after();
         const bool last_of_hp = !more || newhead;
@@ -877,10 +885,13 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
         const uint32_t aG = slot_addr(2 * qgp), aQ = slot_addr(2 * qgp + 1);
         // ---- dA_g = V G_g^T (into S's columns once S_g is read, or, token-wise,
         // into its own columns once dA_{g-1} is read)
-        if (c == 0) wfull(2 * kvp + 1, 0x903);
-        wfull(2 * qgp, 0x904);
-        if (!TW) wt(sd_free_s, g & 1, 0x905);
-        else if (g > 0) wt(sd_free_da, (g - 1) & 1, 0x905);
+        {
+          const BarPhase gf{full_bar(2 * qgp), (fpar >> (2 * qgp)) & 1u};
+          const BarPhase three[3] = {gf, c == 0 ? BarPhase{full_bar(2 * kvp + 1), (fpar >> (2 * kvp + 1)) & 1u} : gf,
+                                     !TW ? BarPhase{sd_free_s, g & 1u} : g > 0 ? BarPhase{sd_free_da, (g - 1) & 1u} : gf};
+          ok = ok && mbar_wait_warp_all(three, abort_flag, a.ws, 0x904);
+          fpar ^= (1u << (2 * qgp)) | (c == 0 ? 1u << (2 * kvp + 1) : 0u);
+        }
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
@@ -893,8 +904,11 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
           if (c == C::NCH - 1) umma_commit(empty_bar(2 * kvp + 1));  // last dA: V free
         }
         // ---- [dV | qbar] += A [G_g | Q_g]
-        wt(a_full, g & 1, 0x906);
-        if (c == 0 && li > 0) wt(acc_empty, (li - 1) & 1, 0x907);
+        {
+          const BarPhase af{a_full, g & 1u};
+          const BarPhase both[2] = {af, c == 0 && li > 0 ? BarPhase{acc_empty, uint32_t(li - 1) & 1u} : af};
+          ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x906);
+        }
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
@@ -910,9 +924,12 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
         if (g + 1 < nchunks) {
           const uint32_t gn = g + 1;
           const int lin = int(gn / C::NCH), cn = int(gn % C::NCH);
-          if (cn == 0) wfull(2 * tok_kv_pair(lin), 0x908);
-          wfull(2 * tok_qg_pair(lin, cn) + 1, 0x909);
-          wt(TW ? sd_free_s : sd_free_da, g & 1, 0x90A);  // S's columns read
+          const int sk = 2 * tok_kv_pair(lin), sq = 2 * tok_qg_pair(lin, cn) + 1;
+          const BarPhase qf{full_bar(sq), (fpar >> sq) & 1u};
+          const BarPhase three[3] = {qf, cn == 0 ? BarPhase{full_bar(sk), (fpar >> sk) & 1u} : qf,
+                                     {TW ? sd_free_s : sd_free_da, g & 1u}};  // S's columns read
+          ok = ok && mbar_wait_warp_all(three, abort_flag, a.ws, 0x909);
+          fpar ^= (1u << sq) | (cn == 0 ? 1u << sk : 0u);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) issue_S(gn);

@@ -274,10 +274,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = mbar_wait_warp(q_full, hc & 1, abort_flag, a.ws, 0x203);
             if (!ok) break;
           }
-          ok = mbar_wait_warp(s_empty, li & 1, abort_flag, a.ws, 0x204);
-          if (!ok) break;
           const int s = int(e % C::NSLOT);
-          ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x205);
+          const BarPhase both[2] = {{s_empty, uint32_t(li) & 1u}, {ring_full(s), (e / C::NSLOT) & 1}};
+          ok = mbar_wait_warp_all(both, abort_flag, a.ws, 0x204);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -292,18 +291,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           if ((li + 2 >= ntiles || nxt.qk != q_now) && elect_one()) umma_commit(q_empty);
         }
         // aggregation of tile li
-        ok = mbar_wait_warp(w_full, li & 1, abort_flag, a.ws, 0x206);
-        if (!ok) break;
         const int s = int(e % C::NSLOT);
-        ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0x207);
-        if (!ok) break;
         // segment sc accumulates into buffer sc % NOB, free once the softmax
         // warps have stored the segment that used it last
         const int ob = sc % C::NOB;
-        if (cur.seg_first && sc >= C::NOB) {
-          ok = mbar_wait_warp(o_empty_of(ob), uint32_t((sc / C::NOB) - 1) & 1u, abort_flag, a.ws, 0x208);
-          if (!ok) break;
-        }
+        const BarPhase w{w_full, uint32_t(li) & 1u};
+        const BarPhase three[3] = {w, {ring_full(s), (e / C::NSLOT) & 1},
+                                   cur.seg_first && sc >= C::NOB
+                                       ? BarPhase{o_empty_of(ob), uint32_t((sc / C::NOB) - 1) & 1u}
+                                       : w};
+        ok = mbar_wait_warp_all(three, abort_flag, a.ws, 0x206);
+        if (!ok) break;
         tc_fence_after();
         const uint64_t dV = sdesc_add(dV0, uint32_t(s) * C::KV_TILE);
         const uint32_t ocol = tmem + C::O_COL + uint32_t(ob * C::O_COLS);
@@ -386,7 +384,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           cur.peek_next(t0n, nn, hn);
           lse_nxt = row < nn ? lse_in[(t0n + row) * a.H + hn] : 0.f;
         }
-        ok = wwait(s_full, li & 1, 0x301);
+        if (MODE == kFused && li > 0) {  // the scores, and the other warpgroup has read the last tile's statistics
+          const BarPhase both[2] = {{s_full, uint32_t(li) & 1u}, {st_used, uint32_t(li - 1) & 1u}};
+          ok = mbar_wait_warp_all(both, abort_flag, a.ws, 0x301);
+        } else {
+          ok = wwait(s_full, li & 1, 0x301);
+        }
         if (!ok) break;
         tc_fence_after();
         float v[C::HALF];
@@ -443,14 +446,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             f = ex2((m - M) * c2) * rcp_approx(Z);
           } else {
             // exchange (max, sum) with the other warpgroup's thread of this token
-            if (li > 0) {
-              ok = wwait(st_used, (li - 1) & 1, 0x304);
-              if (!ok) break;
-            }
             stats[sw * T + row] = make_float2(m, z);
             __syncwarp();
             if (lane == 0) mbar_arrive(st_ready);
-            ok = wwait(st_ready, li & 1, 0x305);
+            // with it: the last aggregation has read the weights
+            const BarPhase sr{st_ready, uint32_t(li) & 1u};
+            const BarPhase both[2] = {sr, li > 0 ? BarPhase{w_empty, uint32_t(li - 1) & 1u} : sr};
+            ok = mbar_wait_warp_all(both, abort_flag, a.ws, 0x305);
             if (!ok) break;
             const float2 o = stats[(1 - sw) * T + row];
             __syncwarp();
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else {
           exp2_shift<C::HALF>(v, c2, valid ? lse_cur * 1.4426950408889634f : INFINITY);
         }
-        if (li > 0) {
+        if (MODE != kFused && li > 0) {
           ok = wwait(w_empty, (li - 1) & 1, 0x302);
           if (!ok) break;
         }

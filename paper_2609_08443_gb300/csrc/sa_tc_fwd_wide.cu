@@ -273,7 +273,10 @@ __global__ void __launch_bounds__(kWThreads, 1)
           prev_q = ws_.qk;
         }
         const int s = li % C::NK;
-        wt(kfull(s), uint32_t(li / C::NK) & 1u, 0x222);
+        // K, and (after the first tile) the softmax warps hold the last scores
+        const BarPhase kf{kfull(s), uint32_t(li / C::NK) & 1u};
+        const BarPhase both[2] = {kf, li > 0 ? BarPhase{s_empty, uint32_t(li - 1) & 1u} : kf};
+        ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x222);
         if (!ok) return;
         tc_fence_after();
         if (elect_one()) {
@@ -294,10 +297,11 @@ __global__ void __launch_bounds__(kWThreads, 1)
         ws_.next();
       };
       auto issue_O = [&](int li) {  // wo is at tile li
-        wt(w_full, uint32_t(li) & 1u, 0x223);
         const int s = li % C::NV;
-        wt(vfull(s), uint32_t(li / C::NV) & 1u, 0x224);
-        if (wo.seg_first && sc > 0) wt(o_empty, uint32_t(sc - 1) & 1u, 0x225);
+        const BarPhase w{w_full, uint32_t(li) & 1u};
+        const BarPhase three[3] = {w, {vfull(s), uint32_t(li / C::NV) & 1u},
+                                   wo.seg_first && sc > 0 ? BarPhase{o_empty, uint32_t(sc - 1) & 1u} : w};
+        ok = ok && mbar_wait_warp_all(three, abort_flag, a.ws, 0x223);
         if (!ok) return;
         tc_fence_after();
         if (elect_one()) {
@@ -326,10 +330,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
       };
       issue_S(0);
       for (int li = 0; li < ntiles && ok; ++li) {
-        if (li + 1 < ntiles) {
-          wt(s_empty, uint32_t(li) & 1u, 0x226);  // the softmax warps hold S(li)
-          if (ok) issue_S(li + 1);
-        }
+        if (li + 1 < ntiles) issue_S(li + 1);
         if (ok) issue_O(li);
       }
       if (elect_one()) umma_commit(drain);  // no UMMA may still run when TMEM is released
@@ -356,8 +357,20 @@ __global__ void __launch_bounds__(kWThreads, 1)
     };
     int seg_idx = 0;
     for (int li = 0; li < ntiles && ok; ++li) {
-      ok = wwait(s_full, uint32_t(li) & 1u, 0x321);
-      if (!ok) break;
+      // the scores and, for the exchange below, the readers of tile li-2 in both CTAs
+      const int b = li & 1;
+      {
+        const uint32_t p2 = uint32_t((li - 2) >> 1) & 1u;
+        const bool t0 = mbar_try_wait(s_full, uint32_t(li) & 1u);
+        const bool t1 = li < 2 || mbar_try_wait(x_free(b), p2);
+        const bool t2 = li < 2 || mbar_try_wait_cluster(r_free(b), p2);
+        if (!__all_sync(0xffffffffu, t0 && t1 && t2)) {
+          ok = wwait(s_full, uint32_t(li) & 1u, 0x321);
+          if (ok && li >= 2) ok = wwait(x_free(b), p2, 0x322);
+          if (ok && li >= 2) ok = wwait_cl(r_free(b), p2, 0x323);
+          if (!ok) break;
+        }
+      }
       tc_fence_after();
       float v[C::GP];
       tmem_ld32(tmem + lane_off + C::S_COL + g * C::GP, v);
@@ -370,21 +383,21 @@ __global__ void __launch_bounds__(kWThreads, 1)
       const float m = row_max<C::GP>(v);
       const float z = exp2_shift_sum<C::GP>(v, c2, m * c2);
       // this thread's partial into this CTA's exchange buffer and the peer's
-      const int b = li & 1;
-      if (li >= 2) {
-        ok = wwait(x_free(b), uint32_t((li - 2) >> 1) & 1u, 0x322);  // this CTA's readers of tile li-2
-        if (!ok) break;
-        ok = wwait_cl(r_free(b), uint32_t((li - 2) >> 1) & 1u, 0x323);  // the peer's readers of tile li-2
-        if (!ok) break;
-      }
       const float2 part = make_float2(m, z);
       X[(b * C::NPART + slot) * T + row] = part;
       st_async_f2(x_peer + uint32_t(((b * C::NPART + slot) * T + row) * 8), part, mapa_shared(x_full(b), peer));
       __syncwarp();
       if (lane == 0) mbar_arrive(x_full(b));
       if (warp == kWSoft0 && lane == 0) mbar_arrive_expect_tx(x_full(b), 4u * T * 8u);
-      ok = wwait_cl(x_full(b), uint32_t(li >> 1) & 1u, 0x324);
-      if (!ok) break;
+      {  // the partials and, for the weights below, O(li-1) has read the last ones
+        const bool t0 = mbar_try_wait_cluster(x_full(b), uint32_t(li >> 1) & 1u);
+        const bool t1 = li == 0 || mbar_try_wait(w_empty, uint32_t(li - 1) & 1u);
+        if (!__all_sync(0xffffffffu, t0 && t1)) {
+          ok = wwait_cl(x_full(b), uint32_t(li >> 1) & 1u, 0x324);
+          if (ok && li > 0) ok = wwait(w_empty, uint32_t(li - 1) & 1u, 0x325);
+          if (!ok) break;
+        }
+      }
       // the token's (max, sum) over all 512 prototypes, partials in slot order
       float2 pp[C::NPART];
 #pragma unroll
@@ -410,10 +423,6 @@ __global__ void __launch_bounds__(kWThreads, 1)
       // natural log of Z through the log2 unit (Z lies in [1, 512])
       if (rank == 0 && g == 0 && valid && lse_out)
         lse_out[(cur.tok0 + row) * a.H + cur.h] = M * a.scale + __log2f(Z) * 0.6931471805599453f;
-      if (li > 0) {
-        ok = wwait(w_empty, uint32_t(li - 1) & 1u, 0x325);  // O(li-1) has read the weights
-        if (!ok) break;
-      }
       // weights -> shared memory, [PS/64 blocks][128 tokens][64 prototypes], 128-byte swizzle:
       // warpgroup g fills block g
       uint8_t* wrow = smem + C::OFF_W + g * (T * 128) + row * 128;

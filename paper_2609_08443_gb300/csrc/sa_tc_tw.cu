@@ -219,10 +219,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = mbar_wait_warp(q_full, hc & 1, abort_flag, a.ws, 0xA03);
             if (!ok) break;
           }
-          ok = mbar_wait_warp(s_empty, li & 1, abort_flag, a.ws, 0xA04);
-          if (!ok) break;
           const int s = int(e % C::NSLOT);
-          ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA05);
+          const BarPhase both[2] = {{s_empty, uint32_t(li) & 1u}, {ring_full(s), (e / C::NSLOT) & 1}};
+          ok = mbar_wait_warp_all(both, abort_flag, a.ws, 0xA04);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -236,15 +235,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           if ((li + 2 >= ntiles || nxt.qk != q_now) && elect_one()) umma_commit(q_empty);
         }
         // O[m-tile] += A[m-tile] V over the tile's 128 tokens, 16 per step
-        ok = mbar_wait_warp(w_full, li & 1, abort_flag, a.ws, 0xA06);
-        if (!ok) break;
         const int s = int(e % C::NSLOT);
-        ok = mbar_wait_warp(ring_full(s), (e / C::NSLOT) & 1, abort_flag, a.ws, 0xA07);
+        const BarPhase w{w_full, uint32_t(li) & 1u};
+        const BarPhase three[3] = {w, {ring_full(s), (e / C::NSLOT) & 1},
+                                   cur.seg_first && sc > 0 ? BarPhase{o_empty, uint32_t(sc - 1) & 1u} : w};
+        ok = mbar_wait_warp_all(three, abort_flag, a.ws, 0xA06);
         if (!ok) break;
-        if (cur.seg_first && sc > 0) {
-          ok = mbar_wait_warp(o_empty, (sc - 1) & 1, abort_flag, a.ws, 0xA08);
-          if (!ok) break;
-        }
         tc_fence_after();
         if (elect_one()) {
           const uint32_t vaddr = sRing + s * C::KV_TILE;
