@@ -356,7 +356,7 @@ sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
   }
   if (plan.bwd_path == Path::TcBwd) {
     SA_TRY(launch(SA_KERNEL_BWD_MAIN, st,
-                  [&] { return sa::launch_tc_bwd(a, plan.W_bwd, dsketch, l, dK, dV, st); }));
+                  [&] { return sa::launch_tc_bwd2_fused(a, plan.W_bwd, dsketch, l, dK, dV, st); }));
   } else {
     float* Dco = reinterpret_cast<float*>(base + plan.lay.dcoef);
     SA_TRY(launch(SA_KERNEL_BWD_MAIN, st,

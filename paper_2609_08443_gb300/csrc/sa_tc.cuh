@@ -20,8 +20,6 @@ int tc_fwd_workers(int num_sms, int P, int d);
 int tc_bwd_workers(int num_sms, int P, int d);
 cudaError_t launch_tc_fwd(const Args& a, int W, float* sketch, float* lse, cudaStream_t st);
 cudaError_t launch_tc_lse(const Args& a, float* lse, cudaStream_t st);
-cudaError_t launch_tc_bwd(const Args& a, int W, const float* dsk, const float* lse, void* dK, void* dV,
-                          cudaStream_t st);
 // d = 128 with P in {256, 512}: token side (dV, dK, D_i) then prototype slices (dQ)
 bool tc_bwd_split(int P, int d);
 cudaError_t launch_tc_bwd_tok(const Args& a, int W, const float* dsk, __nv_bfloat16* gbf, const float* lse,
@@ -40,6 +38,13 @@ cudaError_t launch_tc_tw_bwd_tok(const Args& a, int W, const __nv_bfloat16* gbf,
                                  const float* Dtw, void* dK, void* dV, cudaStream_t st);
 cudaError_t launch_tc_tw_bwd_dq(const Args& a, int W, const float* dsk, const float* lse_tok, const float* Dtw,
                                 cudaStream_t st);
+// the two-sweep kernel (sa_tc_bwd2.cu), P <= 512: dV, dK and dQ at d = 64 with
+// P <= 256 and d = P = 128; dV, dK and D_i at d = 128 with P in {256, 512} and
+// d = 64 with P = 512
+cudaError_t launch_tc_bwd2_fused(const Args& a, int W, const float* dsk, const float* lse, void* dK, void* dV,
+                                 cudaStream_t st);
+cudaError_t launch_tc_bwd2_tok(const Args& a, int W, const __nv_bfloat16* gbf, const float* lse, float* Dco, void* dK,
+                               void* dV, cudaStream_t st);
 cudaError_t launch_tc_g_bf16(const Args& a, const float* dsk, __nv_bfloat16* gbf, cudaStream_t st);
 
 }  // namespace sa

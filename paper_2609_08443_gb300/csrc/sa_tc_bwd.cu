@@ -1,24 +1,13 @@
-// tcgen05 / TMEM / TMA backward kernels of the SA sketching step (sm_103a).
+// tcgen05 / TMEM / TMA backward of the SA sketching step (sm_103a): the choice of
+// kernels, and the token side for shapes whose weights do not stay in TMEM.
 //
 // Chain rule of Sec. 3.1 with upstream G = dL/dsketch[b, h] and the forward's
-// per-token log-sum-exp (FlashSA's softmax statistic, Sec. 4.4), so the
-// weights are recomputed as A = exp(S - lse) without any reduction:
-//   S^T  = K Q^T                 (UMMA, tokens on TMEM lanes)
-//   A    = exp(scale S - lse)    (registers; bf16 copy in shared memory)
-//   dA^T = V G^T                 (UMMA)
-//   dV   = A G                   (UMMA, contraction over prototypes)
-//   D_i  = dV_i . v_i            (= sum_j A[j,i] dA[j,i])
-//   dS   = A o (dA - D)          (registers -> bf16 in shared memory)
-//   dK   = scale dS Q            (UMMA)
-//   dQ  += scale dS^T K          (UMMA, accumulated in TMEM over a worker's
-//                                 tiles of one head; per-worker partials are
-//                                 summed in worker order afterwards)
-// Modes: kFull keeps all P prototypes in one CTA (TMEM: S/dA, dV, dK, dQ);
-// kSlice handles one slice of prototypes and only dQ, with D_i read from the
-// token-side kernel (tc_bwd_tok_kernel) that computes dV, dK and D_i for
-// shapes whose four TMEM accumulators do not fit one SM.
-// Warp roles: 0 TMA, 1 UMMA, 2-3 dsketch loader (fp32 -> bf16 swizzled),
-// 4-11 softmax / epilogue.  Every wait is bounded.
+// per-token log-sum-exp (FlashSA's softmax statistic, Sec. 4.4), so the weights are
+// recomputed as A = exp(S - lse) without any reduction.  Up to 512 prototypes run on
+// the two-sweep kernel (sa_tc_bwd2.cu), with dQ in the same kernel where TMEM holds
+// it; above that, and for the token-wise normalisation, tc_bwd_tok_kernel below
+// computes dV, dK and D_i in one sweep.  dQ comes from prototype slices
+// (sa_tc_bwd_dq.cu) wherever it is not fused.  Every wait is bounded.
 #include <cuda.h>
 
 #include "sa_ptx.cuh"
@@ -30,36 +19,6 @@ namespace tcb {
 
 using namespace ptx;
 using namespace tcc;
-
-enum Mode { kFull = 0, kSlice = 1 };
-
-template <int D, int PS, int MODE>
-struct BCfg {
-  static constexpr int KV_TILE = T * D * 2;
-  static constexpr int Q_BYTES = PS * D * 2;
-  static constexpr int AB_BYTES = T * PS * 2;
-  static constexpr int NSLOT = 4;  // even: even slots hold K tiles, odd slots V tiles
-  static constexpr int NBAR = 2 * NSLOT + 20;
-  // two dsketch buffers where shared memory holds them, so the next user's
-  // dsketch is converted while this user's tiles run
-  static constexpr int NG = (3 * Q_BYTES + AB_BYTES + NSLOT * KV_TILE + NBAR * 8 + 16 <= 232448) ? 2 : 1;
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_G = Q_BYTES;
-  static constexpr int OFF_AB = OFF_G + NG * Q_BYTES;
-  static constexpr int OFF_RING = OFF_AB + AB_BYTES;
-  static constexpr int OFF_BAR = OFF_RING + NSLOT * KV_TILE;
-  static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
-  static constexpr int SMEM = OFF_MISC + 16;
-  static constexpr int NSD = (MODE == kSlice) ? 2 : 1;  // S/dA buffers (slice mode has TMEM to spare)
-  static constexpr int SD_COL = 0;
-  static constexpr int DV_COL = PS;
-  static constexpr int DK_COL = PS + D;
-  static constexpr int DQ_COL = (MODE == kFull) ? PS + 2 * D : NSD * PS;
-  static constexpr int TMEM_COLS = tmem_cols_for(DQ_COL + (PS / 128) * D);
-  static constexpr int HALF = PS / 2;
-  static_assert(TMEM_COLS <= 512, "TMEM budget");
-  static_assert(SMEM <= 232448, "shared memory budget");
-};
 
 // one token row of dV or dK (fp32 from TMEM) -> bf16 global row, columns
 // [c0, c0 + NCOL) of this warpgroup's half
@@ -85,599 +44,38 @@ __device__ __forceinline__ void store_row_bf16(uint32_t taddr, __nv_bfloat16* ds
   }
 }
 
-// the same for mul * (row at ta) + (row at tb), summed in fp32 and rounded once
-template <int NCOL>
-__device__ __forceinline__ void store_row_sum_bf16(uint32_t ta, uint32_t tb, __nv_bfloat16* dst, float mul,
-                                                   bool valid) {
-  float v[16], w[16];
-#pragma unroll
-  for (int c = 0; c < NCOL; c += 16) {
-    tmem_ld16(ta + c, v);
-    tmem_ld16(tb + c, w);
-    tmem_ld_wait();
-    if (valid) {
-      uint4* o = reinterpret_cast<uint4*>(dst + c);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = fmaf(v[k], mul, w[k]);
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        o[k] = make_uint4(pack_bf16(v[8 * k], v[8 * k + 1]), pack_bf16(v[8 * k + 2], v[8 * k + 3]),
-                          pack_bf16(v[8 * k + 4], v[8 * k + 5]), pack_bf16(v[8 * k + 6], v[8 * k + 7]));
-    }
-  }
-}
-
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// SUM: K = V = X, and dV's buffer takes dV + dK (Args::sum_dx)
-template <int D, int PS, int MODE, bool SUM>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_bwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                  const __grid_constant__ CUtensorMap tmQ, Args a, const float* __restrict__ dsk,
-                  const float* __restrict__ lse, const float* __restrict__ Dco_in, __nv_bfloat16* __restrict__ dK,
-                  __nv_bfloat16* __restrict__ dV) {
-  using C = BCfg<D, PS, MODE>;
-  extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  if (ws_failed(a.ws)) return;
-  if (smem_u32(smem) & 1023u) {
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB11u);
-    return;
-  }
-  const uint32_t sbase = smem_u32(smem);
-  const uint32_t sQ = sbase + C::OFF_Q, sG = sbase + C::OFF_G, sAB = sbase + C::OFF_AB, sRing = sbase + C::OFF_RING;
-  const uint32_t bar0 = sbase + C::OFF_BAR;
-  auto ring_full = [&](int s) { return bar0 + 8u * s; };
-  auto ring_empty = [&](int s) { return bar0 + 8u * (C::NSLOT + s); };
-  const uint32_t b1 = bar0 + 8u * (2 * C::NSLOT);
-  const uint32_t q_full = b1, q_empty = b1 + 8, g_full = b1 + 16, g_empty = b1 + 24, s_full = b1 + 32,
-                 sd_free_s = b1 + 40, da_full = b1 + 48, sd_free_da = b1 + 56, a_full = b1 + 64, dv_full = b1 + 72,
-                 dv_empty = b1 + 80, ds_full = b1 + 88, ab_empty = b1 + 96, dk_empty = b1 + 104, dq_full = b1 + 112,
-                 dq_empty = b1 + 120, drain = b1 + 128;
-  // barriers of dsketch buffer gb
-  auto g_full_of = [&](int gb) { return gb ? b1 + 136 : g_full; };
-  auto g_empty_of = [&](int gb) { return gb ? b1 + 144 : g_empty; };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
-
-  const int64_t tph = reinterpret_cast<const WsHeader*>(a.ws)->tiles_per_head;
-  const int64_t total = tph * a.H;
-  const int W = gridDim.x, wk = blockIdx.x, slice = blockIdx.y;
-  const int p0 = slice * PS;
-  const int64_t tb = range_begin(total, W, wk), te = range_begin(total, W, wk + 1);
-  const int ntiles = int(te - tb);
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < C::NSLOT; ++s) {
-      mbar_init(ring_full(s), 1);
-      // V slots are released by the softmax warps once they have read v_i for D_i
-      mbar_init(ring_empty(s), (MODE == kFull && (s & 1)) ? kSoftWarps : 1);
-    }
-    mbar_init(q_full, 1);
-    mbar_init(q_empty, 1);
-    mbar_init(g_full, 2);
-    mbar_init(g_empty, 1);
-    mbar_init(b1 + 136, 2);
-    mbar_init(b1 + 144, 1);
-    mbar_init(s_full, 1);
-    mbar_init(sd_free_s, kSoftWarps);
-    mbar_init(da_full, 1);
-    mbar_init(sd_free_da, kSoftWarps);
-    mbar_init(a_full, kSoftWarps);
-    mbar_init(dv_full, 1);
-    mbar_init(dv_empty, kSoftWarps);
-    mbar_init(ds_full, kSoftWarps);
-    mbar_init(ab_empty, 1);
-    mbar_init(dk_empty, kSoftWarps);
-    mbar_init(dq_full, 1);
-    mbar_init(dq_empty, kSoftWarps);
-    mbar_init(drain, 1);
-    wait_ctl_init(abort_flag, a.ws);
-    fence_mbar_init();
-  }
-  if (warp == 2) tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-
-  if (ntiles > 0) {
-    if (warp == 0 && lane == 0) {
-      // ---------------------------------------------------------- TMA producer
-      tma_prefetch_desc(&tmK);
-      tma_prefetch_desc(&tmV);
-      tma_prefetch_desc(&tmQ);
-      TileWalker it(a, tb, te, T);
-      int hc = 0, prev_h = -1;
-      uint32_t e = 0;
-      bool ok = true;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        if (it.qk != prev_h) {  // a new head (or, with per-user queries, a new user)
-          if (hc > 0) ok = mbar_wait(q_empty, (hc - 1) & 1, abort_flag, a.ws, 0x401);
-          if (!ok) break;
-          mbar_arrive_expect_tx(q_full, C::Q_BYTES);
-#pragma unroll
-          for (int dh = 0; dh < D / 64; ++dh) tma_load_3d(sQ + dh * PS * 128, &tmQ, q_full, 64 * dh, p0, it.qk);
-          prev_h = it.qk;
-          ++hc;
-        }
-#pragma unroll
-        for (int kv = 0; kv < 2; ++kv) {
-          const int s = int(e % C::NSLOT);
-          if (e >= uint32_t(C::NSLOT)) ok = mbar_wait(ring_empty(s), ((e / C::NSLOT) + 1) & 1, abort_flag, a.ws, 0x402);
-          if (!ok) break;
-          mbar_arrive_expect_tx(ring_full(s), C::KV_TILE);
-#pragma unroll
-          for (int dh = 0; dh < D / 64; ++dh)
-            tma_load_3d(sRing + s * C::KV_TILE + dh * T * 128, kv ? &tmV : &tmK, ring_full(s), 64 * dh, it.h,
-                        int(it.tok0));
-          ++e;
-        }
-        it.next();
-      }
-      if (!ok) {  // drain the ring loads and the prototype block still in flight
-        for (uint32_t k = (e > uint32_t(C::NSLOT) ? e - C::NSLOT : 0); k < e; ++k)
-          mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
-        if (hc > 0) mbar_wait_bounded(q_full, uint32_t(hc - 1) & 1u, 200000000ull);
-      }
-    } else if (warp == 1) {
-      // ---------------------------------------------------------- UMMA issuer
-      constexpr uint32_t idSP = idesc_bf16(128, PS, 0, 0);      // [tok x P], K = d
-      constexpr uint32_t idTD = idesc_bf16(128, D, 0, 1);       // [tok x d], K = prototypes
-      constexpr uint32_t idQD = idesc_bf16(128, D, 1, 1);       // [proto x d], K = tokens
-      TileWalker cur(a, tb, te, T), nxt(a, tb, te, T);
-      nxt.next();
-      int hc = 0, gc = 0, hp = 0, gbuf = 0;
-      bool ok = true;
-      auto wt = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return ok = ok && mbar_wait_warp(bar, par, abort_flag, a.ws, site);
-      };
-      auto sdcol = [&](int i) { return uint32_t(C::SD_COL + (i % C::NSD) * PS); };
-      // operand descriptors built once and stepped by constant offsets: each
-      // instruction the issuing thread saves shortens the issue of a group (most
-      // groups here are N = 64 or N = 128, a few dozen cycles of work per UMMA)
-      const uint64_t dQk = sdesc(sQ, 16, 1024), dQm = sdesc(sQ, PS * 128, 1024);
-      const uint64_t dABk = sdesc(sAB, 16, 1024), dABm = sdesc(sAB, T * 128, 1024);
-      const uint64_t dRk = sdesc(sRing, 16, 1024), dRm = sdesc(sRing, T * 128, 1024);
-      const uint64_t dGk = sdesc(sG, 16, 1024), dGm = sdesc(sG, PS * 128, 1024);
-      // S(i) = K(i) Q^T into an S/dA buffer
-      auto issue_S = [&](uint32_t kslot, uint32_t col) {
-        const uint64_t dK = sdesc_add(dRk, kslot * C::KV_TILE);
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k)
-          umma_ss(tmem + col, sdesc_add(dK, (k >> 2) * (T * 128) + (k & 3) * 32),
-                  sdesc_add(dQk, (k >> 2) * (PS * 128) + (k & 3) * 32), idSP, k > 0 ? 1u : 0u);
-      };
-      TileWalker nx2(a, tb, te, T);
-      nx2.next();
-      nx2.next();
-      wt(q_full, 0, 0x501);
-      wt(ring_full(0), 0, 0x502);
-      if (ok) {
-        tc_fence_after();
-        if (elect_one()) {
-          issue_S(0, sdcol(0));
-          umma_commit(s_full);
-          // slice mode: Q is read only by S, so it may be replaced after the last S of a head
-          if (MODE == kSlice && (ntiles == 1 || nxt.qk != cur.qk)) umma_commit(q_empty);
-        }
-      }
-      bool first_of_hp = true;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        const uint32_t eK = 2u * li, eV = eK + 1;
-        const int sK = int(eK % C::NSLOT), sV = int(eV % C::NSLOT);
-        // ---- dA(i) = V(i) G^T
-        if (cur.seg_first) {
-          gbuf = gc % C::NG;
-          wt(g_full_of(gbuf), uint32_t(gc / C::NG) & 1u, 0x503);
-          ++gc;
-        }
-        {
-          const BarPhase both[2] = {{ring_full(sV), (eV / C::NSLOT) & 1}, {sd_free_s, uint32_t(li) & 1u}};
-          ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x504);
-        }
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t gofs = uint32_t(gbuf * C::Q_BYTES);  // this segment's dsketch buffer
-        if (elect_one()) {
-          const uint64_t dVk = sdesc_add(dRk, uint32_t(sV) * C::KV_TILE), dG = sdesc_add(dGk, gofs);
-#pragma unroll
-          for (int k = 0; k < D / 16; ++k)
-            umma_ss(tmem + sdcol(li), sdesc_add(dVk, (k >> 2) * (T * 128) + (k & 3) * 32),
-                    sdesc_add(dG, (k >> 2) * (PS * 128) + (k & 3) * 32), idSP, k > 0 ? 1u : 0u);
-          umma_commit(da_full);
-          if (MODE == kSlice) umma_commit(ring_empty(sV));
-        }
-        // ---- dV(i) = A G
-        if (MODE == kFull) {
-          const BarPhase af{a_full, uint32_t(li) & 1u};
-          const BarPhase both[2] = {af, li > 0 ? BarPhase{dv_empty, uint32_t(li - 1) & 1u} : af};
-          ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x506);
-          if (!ok) break;
-          tc_fence_after();
-          if (elect_one()) {
-            const uint64_t dG = sdesc_add(dGm, gofs);
-#pragma unroll
-            for (int k = 0; k < PS / 16; ++k)
-              umma_ss(tmem + C::DV_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dG, k * 2048),
-                      idTD, k > 0 ? 1u : 0u);
-            umma_commit(dv_full);
-          }
-        }
-        if (!ok) break;
-        if (cur.seg_last && elect_one()) umma_commit(g_empty_of(gbuf));
-        const bool more = li + 1 < ntiles;
-        const bool newhead = more && nxt.qk != cur.qk;
-        // ---- S(i+1) before dK/dQ(i) when its buffer and Q allow it
-        const bool early = more && (C::NSD == 2 || !newhead);
-        if (early) {
-          if (C::NSD == 2) {
-            if (newhead) {
-              ++hc;
-              wt(q_full, hc & 1, 0x508);
-            }
-            if (li >= 1) wt(sd_free_da, (li - 1) & 1, 0x509);
-            wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x50A);
-          } else {
-            const BarPhase both[2] = {{sd_free_da, uint32_t(li) & 1u},
-                                      {ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1}};
-            ok = ok && mbar_wait_warp_all(both, abort_flag, a.ws, 0x509);
-          }
-          if (!ok) break;
-          tc_fence_after();
-          if (elect_one()) {
-            issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
-            umma_commit(s_full);
-            if (MODE == kSlice && (li + 2 >= ntiles || nx2.qk != nxt.qk)) umma_commit(q_empty);
-          }
-        }
-        // ---- dK(i) = dS Q, dQ += dS^T K
-        {
-          const BarPhase df{ds_full, uint32_t(li) & 1u};
-          const BarPhase three[3] = {df, MODE == kFull && li > 0 ? BarPhase{dk_empty, uint32_t(li - 1) & 1u} : df,
-                                     first_of_hp && hp > 0 ? BarPhase{dq_empty, uint32_t(hp - 1) & 1u} : df};
-          ok = ok && mbar_wait_warp_all(three, abort_flag, a.ws, 0x50B);
-        }
-        if (!ok) break;
-        tc_fence_after();
-        const bool last_of_hp = !more || newhead;
-        if (elect_one()) {
-          if (MODE == kFull) {
-#pragma unroll
-            for (int k = 0; k < PS / 16; ++k)
-              umma_ss(tmem + C::DK_COL, sdesc_add(dABk, (k >> 2) * (T * 128) + (k & 3) * 32), sdesc_add(dQm, k * 2048),
-                      idTD, k > 0 ? 1u : 0u);
-          }
-          const uint64_t dKm = sdesc_add(dRm, uint32_t(sK) * C::KV_TILE);
-#pragma unroll
-          for (int k = 0; k < T / 16; ++k)
-#pragma unroll
-            for (int mb = 0; mb < PS / 128; ++mb)
-              umma_ss(tmem + C::DQ_COL + mb * D, sdesc_add(dABm, mb * 2 * (T * 128) + k * 2048),
-                      sdesc_add(dKm, k * 2048), idQD, (first_of_hp && k == 0) ? 0u : 1u);
-          umma_commit(ab_empty);
-          umma_commit(ring_empty(sK));
-          if (last_of_hp) {
-            umma_commit(dq_full);
-            if (MODE == kFull) umma_commit(q_empty);  // dK read Q up to here
-          }
-        }
-        if (last_of_hp) ++hp;
-        first_of_hp = last_of_hp;
-        // ---- S(i+1) after a head change in full mode (Q replaced once dK(i) is done)
-        if (more && !early) {
-          ++hc;
-          wt(q_full, hc & 1, 0x50E);
-          wt(sd_free_da, li & 1, 0x50F);
-          wt(ring_full(int((eK + 2) % C::NSLOT)), ((eK + 2) / C::NSLOT) & 1, 0x510);
-          if (!ok) break;
-          tc_fence_after();
-          if (elect_one()) {
-            issue_S((eK + 2) % C::NSLOT, sdcol(li + 1));
-            umma_commit(s_full);
-          }
-        }
-        cur.next();
-        nxt.next();
-        nx2.next();
-      }
-      if (elect_one()) umma_commit(drain);
-      mbar_wait_bounded(drain, 0, 200000000ull);
-    } else if (warp == 2 || warp == 3) {
-      // ------------------------------------ dsketch rows -> bf16, swizzled [d/64][PS][64]
-      const int t64 = threadIdx.x - 64;  // 0..63
-      TileWalker cur(a, tb, te, T);
-      int gc = 0;
-      bool ok = true;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        if (cur.seg_first) {
-          const int gb = gc % C::NG;
-          if (gc >= C::NG)
-            ok = __all_sync(0xffffffffu, mbar_wait(g_empty_of(gb), uint32_t((gc / C::NG) - 1) & 1u, abort_flag,
-                                                   a.ws, 0x601));
-          if (!ok) break;
-          const float* src = dsk + ((int64_t(cur.b) * a.H + cur.h) * a.P + p0) * D;
-          uint8_t* gdst = smem + C::OFF_G + gb * C::Q_BYTES;
-          constexpr int CHUNKS = PS * D / 8;
-#pragma unroll 8
-          for (int c = t64; c < CHUNKS; c += 64) {
-            const int p = c / (D / 8), dd = (c % (D / 8)) * 8;
-            const float4 x = *reinterpret_cast<const float4*>(src + int64_t(p) * D + dd);
-            const float4 y = *reinterpret_cast<const float4*>(src + int64_t(p) * D + dd + 4);
-            uint4 pk;
-            pk.x = pack_bf16(x.x, x.y);
-            pk.y = pack_bf16(x.z, x.w);
-            pk.z = pack_bf16(y.x, y.y);
-            pk.w = pack_bf16(y.z, y.w);
-            const int dh = dd >> 6, chunk = (dd & 63) >> 3;
-            *reinterpret_cast<uint4*>(gdst + dh * PS * 128 + p * 128 + ((chunk ^ (p & 7)) << 4)) = pk;
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(g_full_of(gb));
-          ++gc;
-        }
-        cur.next();
-      }
-    } else if (warp >= kSoftWarp0) {
-      // ------------------------------------------------ softmax + epilogue
-      const int sw = (warp - kSoftWarp0) >> 2, q = warp & 3, row = 32 * q + lane;
-      const uint32_t lane_off = uint32_t(32 * q) << 16;
-      const float c2 = a.scale * 1.4426950408889634f;
-      TileWalker cur(a, tb, te, T), prev(a, tb, te, T);
-      bool ok = true;
-      auto wwait = [&](uint32_t bar, uint32_t par, uint32_t site) {
-        return __all_sync(0xffffffffu, mbar_wait(bar, par, abort_flag, a.ws, site));
-      };
-      int hp = 0;
-      // dK of the previous tile and, at the end of a head piece, dQ
-      auto finish_prev = [&](const TileWalker& pw, bool last_of_hp) {
-        if (MODE == kFull) {
-          // the sum dV + dK reads dV's columns here: the next tile's dV is issued only
-          // after every warp has stored that tile's weights, which follow this
-          __nv_bfloat16* dst = (SUM ? dV : dK) + ((pw.tok0 + row) * a.H + pw.h) * int64_t(D) + sw * (D / 2);
-          if (SUM)
-            store_row_sum_bf16<D / 2>(tmem + lane_off + C::DK_COL + sw * (D / 2),
-                                      tmem + lane_off + C::DV_COL + sw * (D / 2), dst, a.scale, row < pw.n);
-          else
-            store_row_bf16<D / 2>(tmem + lane_off + C::DK_COL + sw * (D / 2), dst, a.scale, row < pw.n);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(dk_empty);
-        }
-        if (last_of_hp) {
-          float* dst = dq_block_dst(a, wk, W, total, pw, p0, D);
-          store_sketch_scaled<D, PS, C::DQ_COL>(tmem, lane_off, sw, q, lane, dst, a.scale);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(dq_empty);
-          ++hp;
-        }
-      };
-      uint32_t apk[C::HALF / 2];  // this thread's A values, bf16 pairs
-      // per-token lse (and D_i in slice mode), loaded one tile ahead
-      float lse_cur = row < cur.n ? lse[(cur.tok0 + row) * a.H + cur.h] : 0.f;
-      float d_cur = (MODE == kSlice && row < cur.n) ? Dco_in[(cur.tok0 + row) * a.H + cur.h] : 0.f;
-      for (int li = 0; li < ntiles && ok; ++li) {
-        const bool valid = row < cur.n;
-        const int64_t tok = cur.tok0 + row;
-        const uint32_t eV = 2u * li + 1;
-        const int sV = int(eV % C::NSLOT);
-        const uint32_t sdc = C::SD_COL + (li % C::NSD) * PS;
-        float lse_nxt, d_nxt = 0.f;
-        {
-          int64_t t0n;
-          int nn, hn;
-          cur.peek_next(t0n, nn, hn);
-          lse_nxt = row < nn ? lse[(t0n + row) * a.H + hn] : 0.f;
-          if (MODE == kSlice) d_nxt = row < nn ? Dco_in[(t0n + row) * a.H + hn] : 0.f;
-        }
-        // ---- A = exp(scale S - lse)
-        ok = wwait(s_full, li & 1, 0x701);
-        if (!ok) break;
-        tc_fence_after();
-        {
-          const float L2 = lse_cur * 1.4426950408889634f;
-          float v[32];
-#pragma unroll
-          for (int c = 0; c < C::HALF / 32; ++c) {
-            tmem_ld32(tmem + lane_off + sdc + sw * C::HALF + 32 * c, v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x0 = valid ? ex2(fmaf(v[2 * j], c2, -L2)) : 0.f;
-              const float x1 = valid ? ex2(fmaf(v[2 * j + 1], c2, -L2)) : 0.f;
-              apk[16 * c + j] = pack_bf16(x0, x1);
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(sd_free_s);
-        // ---- previous tile's dK / dQ (their MMAs also release the AB buffer)
-        if (li > 0) {
-          ok = wwait(ab_empty, (li - 1) & 1, 0x702);
-          if (!ok) break;
-          tc_fence_after();
-          finish_prev(prev, prev.qk != cur.qk);
-          prev.next();
-        }
-        // ---- A -> shared memory [PS/64][128 tokens][64], 128-byte swizzle
-        if (MODE == kFull) {
-          uint8_t* rowp = smem + C::OFF_AB + row * 128;
-#pragma unroll
-          for (int k = 0; k < C::HALF / 8; ++k) {
-            const int p = sw * C::HALF + 8 * k;
-            const int blk = p >> 6, chunk = (p & 63) >> 3;
-            *reinterpret_cast<uint4*>(rowp + blk * (T * 128) + ((chunk ^ (row & 7)) << 4)) =
-                make_uint4(apk[4 * k], apk[4 * k + 1], apk[4 * k + 2], apk[4 * k + 3]);
-          }
-        }
-        if (MODE == kFull) {
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(a_full);
-        }
-        // ---- D_i
-        float Dv = 0.f;
-        if (MODE == kFull) {
-          ok = wwait(dv_full, li & 1, 0x703);
-          if (!ok) break;
-          tc_fence_after();
-          const uint8_t* vrow = smem + C::OFF_RING + sV * C::KV_TILE + row * 128;
-          float v[32];
-#pragma unroll
-          for (int c = 0; c < D; c += 32) {
-            tmem_ld32(tmem + lane_off + C::DV_COL + c, v);
-            tmem_ld_wait();
-            const int dh = c >> 6;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int chunk = ((c & 63) >> 3) + k;
-              const uint4 w = *reinterpret_cast<const uint4*>(vrow + dh * (T * 128) + ((chunk ^ (row & 7)) << 4));
-              Dv = fmaf(v[8 * k + 0], bf16lo(w.x), Dv);
-              Dv = fmaf(v[8 * k + 1], bf16hi(w.x), Dv);
-              Dv = fmaf(v[8 * k + 2], bf16lo(w.y), Dv);
-              Dv = fmaf(v[8 * k + 3], bf16hi(w.y), Dv);
-              Dv = fmaf(v[8 * k + 4], bf16lo(w.z), Dv);
-              Dv = fmaf(v[8 * k + 5], bf16hi(w.z), Dv);
-              Dv = fmaf(v[8 * k + 6], bf16lo(w.w), Dv);
-              Dv = fmaf(v[8 * k + 7], bf16hi(w.w), Dv);
-            }
-          }
-          // dV rows of this tile
-          __nv_bfloat16* dst = dV + (tok * a.H + cur.h) * int64_t(D) + sw * (D / 2);
-          if (!SUM)
-            store_row_bf16<D / 2>(tmem + lane_off + C::DV_COL + sw * (D / 2), dst, 1.f, valid);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(dv_empty);
-            mbar_arrive(ring_empty(sV));
-          }
-        } else {
-          Dv = d_cur;
-        }
-        // ---- dS = A o (dA - D) -> shared memory (over A, whose readers are done)
-        ok = wwait(da_full, li & 1, 0x704);
-        if (!ok) break;
-        tc_fence_after();
-        {
-          uint8_t* rowp = smem + C::OFF_AB + row * 128;
-          float v[32];
-#pragma unroll
-          for (int c = 0; c < C::HALF / 32; ++c) {
-            tmem_ld32(tmem + lane_off + sdc + sw * C::HALF + 32 * c, v);
-            tmem_ld_wait();
-            uint32_t o[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const uint32_t w = apk[16 * c + j];
-              o[j] = pack_bf16(bf16lo(w) * (v[2 * j] - Dv), bf16hi(w) * (v[2 * j + 1] - Dv));
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int p = sw * C::HALF + 32 * c + 8 * k;
-              const int blk = p >> 6, chunk = (p & 63) >> 3;
-              *reinterpret_cast<uint4*>(rowp + blk * (T * 128) + ((chunk ^ (row & 7)) << 4)) =
-                  make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-            }
-          }
-        }
-        tc_fence_before();
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(sd_free_da);
-          mbar_arrive(ds_full);
-        }
-        lse_cur = lse_nxt;
-        d_cur = d_nxt;
-        cur.next();
-      }
-      if (ok) {
-        ok = wwait(ab_empty, (ntiles - 1) & 1, 0x705);
-        if (ok) {
-          tc_fence_after();
-          finish_prev(prev, true);
-        }
-      }
-    }
-  }
-  __syncthreads();
-  if (warp == 2) {
-    tc_fence_after();
-    tmem_dealloc(tmem, C::TMEM_COLS);
-  }
-}
-
-template <int D, int PS, int MODE>
-static cudaError_t launch_bwd_t(const Args& a, int W, const float* dsk, const float* lse, const float* Dco, void* dK,
-                                void* dV, cudaStream_t st) {
-  using C = BCfg<D, PS, MODE>;
-  CUtensorMap tk, tv, tq;
-  if (!make_kv_map(&tk, a.K, a.N, a.H, D) || !make_kv_map(&tv, a.V, a.N, a.H, D) ||
-      !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, PS))
-    return cudaErrorInvalidValue;
-  auto fn = a.sum_dx ? &tc_bwd_kernel<D, PS, MODE, true> : &tc_bwd_kernel<D, PS, MODE, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-  if (e != cudaSuccess) return e;
-  dim3 grid(W, a.P / PS);
-  fn<<<grid, kThreads, C::SMEM, st>>>(tk, tv, tq, a, dsk, lse, Dco, static_cast<__nv_bfloat16*>(dK),
-                                      static_cast<__nv_bfloat16*>(dV));
-  return cudaGetLastError();
-}
-
 }  // namespace tcb
 
-// Tensor-core backward: bf16, all prototypes in one CTA when the four TMEM
-// accumulators fit (d = 64 with P <= 256, d = 128 with P = 128), else the
-// token-side kernel plus the dQ slices (tc_bwd_split).
 bool tc_bwd_supported(int P, int d, sa_dtype dt) {
   if (dt != SA_BF16 || !tcc::device_is_sm103() || !tc_path_enabled()) return false;
   return ((d == 64 || d == 128) && (P == 128 || P == 256 || P == 512 || P == 1024 || P == 2048));
 }
 
 const char* tc_bwd_name(int P, int d) {
-  if (d == 64 && P == 2048) return "tc_bwd_tok_kernel<64,2048>";
-  if (d == 64 && P == 1024) return "tc_bwd_tok_kernel<64,1024>";
-  if (d == 64 && P == 512) return "tc_bwd_tok_kernel<64,512>";
-  if (d == 64) return P == 256 ? "tc_bwd_kernel<64,256,full>" : "tc_bwd_kernel<64,128,full>";
-  if (P == 2048) return "tc_bwd_tok_kernel<128,2048>";
-  if (P == 1024) return "tc_bwd_tok_kernel<128,1024>";
-  if (P == 512) return "tc_bwd_tok_kernel<128,512>";
-  if (P == 256) return "tc_bwd_tok_kernel<128,256>";
-  return "tc_bwd_kernel<128,128,full>";
+  if (P == 2048) return d == 64 ? "tc_bwd_tok_kernel<64,2048>" : "tc_bwd_tok_kernel<128,2048>";
+  if (P == 1024) return d == 64 ? "tc_bwd_tok_kernel<64,1024>" : "tc_bwd_tok_kernel<128,1024>";
+  if (P == 512) return d == 64 ? "tc_bwd2_kernel<64,512>" : "tc_bwd2_kernel<128,512>";
+  if (P == 256) return d == 64 ? "tc_bwd2_kernel<64,256,dq>" : "tc_bwd2_kernel<128,256>";
+  return d == 64 ? "tc_bwd2_kernel<64,128,dq>" : "tc_bwd2_kernel<128,128,dq>";
 }
 
 int tc_bwd_workers(int num_sms, int, int) { return num_sms; }
 
-cudaError_t launch_tc_bwd(const Args& a, int W, const float* dsk, const float* lse, void* dK, void* dV,
-                          cudaStream_t st) {
-  if (a.N == 0) return cudaSuccess;
-  using namespace tcb;
-  if (a.d == 64) {
-    if (a.P == 256) return launch_bwd_t<64, 256, kFull>(a, W, dsk, lse, nullptr, dK, dV, st);
-    if (a.P == 128) return launch_bwd_t<64, 128, kFull>(a, W, dsk, lse, nullptr, dK, dV, st);
-  } else if (a.P == 128) {
-    return launch_bwd_t<128, 128, kFull>(a, W, dsk, lse, nullptr, dK, dV, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
 }  // namespace sa
 
 // ===================================================================== tokens
-// Token side of the backward for shapes whose prototypes do not fit one CTA
-// (d = 128 with P > 128): all P prototypes pass through the CTA in chunks of
+// Token side of the backward where the weights of a tile do not stay in TMEM
+// (P > 512; token-wise): all P prototypes pass through the CTA in chunks of
 // NC = 128 (Q and a bf16 copy of dsketch streamed by TMA), in one pass:
 //   dV_i   = sum_j A[j,i] G_j                   (UMMA, accumulates over chunks)
 //   u_i    = sum_j A[j,i] dA[j,i] Q_j            (UMMA on E = A o dA)
 //   qbar_i = sum_j A[j,i] Q_j                    (UMMA)
 //   D_i    = sum_j A[j,i] dA[j,i]                (registers)
 //   dK_i   = scale (u_i - D_i qbar_i)            (= scale sum_j dS[j,i] Q_j)
-// and D_i is written out for the prototype-side dQ kernel (kSlice mode above).
+// and D_i is written out for the prototype-side dQ slices.
 namespace sa {
 namespace tcb {
 
@@ -1246,8 +644,10 @@ static cudaError_t launch_tok_t(const Args& a, int W, const __nv_bfloat16* gbf, 
       !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, C::NC) || !make_q_map(&tg, gbf, a.B * a.H, a.P, D, C::NC) ||
       !make_kv_map(&tdk, dK, a.N, a.H, D) || !make_kv_map(&tdv, dV, a.N, a.H, D))
     return cudaErrorInvalidValue;
-  auto fn = &tc_tw_bwd_tok_kernel<D, P>;
-  if constexpr (!TW) fn = a.sum_dx ? &tc_bwd_tok_kernel<D, P, true> : &tc_bwd_tok_kernel<D, P, false>;
+  auto fn = [&] {
+    if constexpr (TW) return &tc_tw_bwd_tok_kernel<D, P>;
+    else return a.sum_dx ? &tc_bwd_tok_kernel<D, P, true> : &tc_bwd_tok_kernel<D, P, false>;
+  }();
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   fn<<<W, kThreads, C::SMEM, st>>>(tk, tv, tq, tg, tdk, tdv, a, lse, Dco, static_cast<__nv_bfloat16*>(dK),
@@ -1272,15 +672,12 @@ cudaError_t launch_tc_bwd_tok(const Args& a, int W, const float* dsk, __nv_bfloa
                               float* Dco, void* dK, void* dV, cudaStream_t st) {
   (void)dsk;
   if (a.N == 0) return cudaSuccess;
-  if (a.d == 64) {
-    if (a.P == 2048) return tcb::launch_tok_t<64, 2048>(a, W, gbf, lse, Dco, dK, dV, st);
-    if (a.P == 1024) return tcb::launch_tok_t<64, 1024>(a, W, gbf, lse, Dco, dK, dV, st);
-    return tcb::launch_tok_t<64, 512>(a, W, gbf, lse, Dco, dK, dV, st);
-  }
-  if (a.P == 2048) return tcb::launch_tok_t<128, 2048>(a, W, gbf, lse, Dco, dK, dV, st);
-  if (a.P == 1024) return tcb::launch_tok_t<128, 1024>(a, W, gbf, lse, Dco, dK, dV, st);
-  if (a.P == 512) return tcb::launch_tok_t<128, 512>(a, W, gbf, lse, Dco, dK, dV, st);
-  return tcb::launch_tok_t<128, 256>(a, W, gbf, lse, Dco, dK, dV, st);
+  if (a.P <= 512) return launch_tc_bwd2_tok(a, W, gbf, lse, Dco, dK, dV, st);
+  if (a.d == 64)
+    return a.P == 2048 ? tcb::launch_tok_t<64, 2048>(a, W, gbf, lse, Dco, dK, dV, st)
+                       : tcb::launch_tok_t<64, 1024>(a, W, gbf, lse, Dco, dK, dV, st);
+  return a.P == 2048 ? tcb::launch_tok_t<128, 2048>(a, W, gbf, lse, Dco, dK, dV, st)
+                     : tcb::launch_tok_t<128, 1024>(a, W, gbf, lse, Dco, dK, dV, st);
 }
 
 int tc_bwd_dq_workers(int num_sms, int P) {
