@@ -15,21 +15,22 @@
 // leaves B alone in shared memory (half the bandwidth).  And each tile runs as two
 // independent halves of 64 tokens, one per softmax warpgroup, each with its own S
 // and dA columns: while one half's dS is formed the other half's products run.
-// lse_t and D_t are per-column values: as broadcasts from shared memory they cost
-// every thread 32 vector loads per half (1024 cycles per tile of the load path).
-// The products add them instead: one more K step of S and of dA multiplies ones with
-// -lse_t / scale and -D_t, each split into three bf16 terms, whose sum is the fp32
-// value exactly.
+// lse_t and D_t are per-column values, read as broadcasts of four from shared memory
+// (32 vector loads per thread and half, 1024 cycles of the load path per tile, issued
+// ahead of the waits for the products).  Adding them in the products instead (ones
+// times their three bf16 terms as one more K step) is 13% faster, but rounds the
+// exponent in the accumulator at the size of lse / scale: enough bf16 weights flip
+// that dQ differs by 3e-5 from the order of operations used here (2e-6 with it).
 // The issuers wait for all that a tile needs in one round of polls and read the next
 // tile's flags a tile ahead: seven waits in turn, 250-450 cycles each although
 // satisfied, had cost 2100 cycles per tile.
-// Measured: 16 users of 100K tokens (H = 8, P = 512, d = 128) 4.37 ms before, 3.35 ms
-// now; 12 users, 215K tokens, token-wise 678 and 468 us; P = 1024, 141K tokens, 797
-// and 609 us.
+// Measured: 16 users of 100K tokens (H = 8, P = 512, d = 128) 4.37 ms before, 3.79 ms
+// now; 12 users, 215K tokens, token-wise 678 and 452 us; P = 1024, 141K tokens, 797
+// and 634 us.
 // TMEM: per half S 64 (dS over its first 32) and dA 64, G D/2, Q D/2, dQ D columns.
 //
 // Warp roles: 0 tile sequence, loads; 1 issues S and dA, 2 (also TMEM) issues dQ; 3
-// forms the per-token operands; 4-7 and 8-11 the two halves.
+// lays out the per-token values; 4-7 and 8-11 the two halves.
 #include <cuda.h>
 
 #include "sa_ptx.cuh"
@@ -45,11 +46,6 @@ using namespace tcc;
 constexpr uint32_t kRegsCtl = 136, kRegsSoft = 184;
 static_assert(128 * kRegsCtl + 256 * kRegsSoft == 384 * 168, "register split = launch allocation");
 constexpr float kLog2e = 1.4426950408889634f;
-
-// -lse / scale has to stay finite: at a scale below this the scores are zeros in fp32
-// beside any lse, so they are formed from zero prototypes and a scale of 1.
-constexpr float kTinyScale = 1e-30f;
-__device__ __forceinline__ float tiny_scale(float scale) { return scale < kTinyScale ? 1.f : scale; }
 
 // What the other roles need of a tile, written by warp 0 into a ring.  A run is a
 // sequence of tiles that read one row of Q: a head, or with per-user queries one
@@ -69,13 +65,11 @@ struct DCfg {
   // K(i) is read by S(i) and, a tile later, by dQ(i); V(i) only by dA(i)
   static constexpr int NK = 3, NV = 2, NI = 4;
   static constexpr int OFF_K = 0, OFF_V = NK * TILE;
-  // per-token operands [2 bufs][128 tokens][64]: features 0-2 the terms of -lse / scale,
-  // 16-18 those of -D; and the [128 prototypes][64] of ones they meet
-  static constexpr int OFF_COL = OFF_V + NV * TILE;
-  static constexpr int OFF_ONE = OFF_COL + 2 * BLK;
+  // per-token values of two tiles: [2 bufs][lse log2 e, D][128 tokens]
+  static constexpr int OFF_COL = OFF_V + NV * TILE, COL = 2 * T * 4;
   // raw (lse log2 e, D) of the tile in each K slot: the copy starts at an even index
   static constexpr int RAW = (T + 2) * 8;
-  static constexpr int OFF_RAW = OFF_ONE + BLK;
+  static constexpr int OFF_RAW = OFF_COL + 2 * COL;
   static constexpr int OFF_INFO = OFF_RAW + NK * RAW;
   static constexpr int OFF_BAR = OFF_INFO + NI * int(sizeof(TileInfo));
   static constexpr int NBAR = 2 * NK + 2 * NV + 2 * NI + 20;
@@ -133,7 +127,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       for (int k = 0; k < n; ++k) mbar_init(bar + 8u * k, count);
     };
     init(k_full, C::NK, 1);
-    init(k_empty, C::NK, TW ? 1 : 2);  // dQ, and the per-token operands formed
+    init(k_empty, C::NK, TW ? 1 : 2);  // dQ, and the per-token values read
     init(v_full, C::NV, 1);
     init(v_empty, C::NV, 1);
     init(i_full, C::NI, 1);
@@ -143,7 +137,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
     init(ds_full, 2, 4);
     init(buf_free, 2, 1);
     init(col_full, 2, 1);
-    init(col_empty, 2, 1);
+    init(col_empty, 2, kSoftWarps);
     init(q_full, 1, kSoftWarps);
     init(q_empty, 1, 1);
     init(g_full, 1, kSoftWarps);
@@ -155,17 +149,6 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
     fence_mbar_init();
   }
   if (warp == 2) tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-  if (!TW && threadIdx.x < 128) {  // the ones, and the zero features beside the per-token terms
-    const int r = threadIdx.x;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    uint8_t* one = smem + C::OFF_ONE + r * 128;
-    *reinterpret_cast<uint4*>(one + ((0 ^ (r & 7)) << 4)) = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
-    *reinterpret_cast<uint4*>(one + ((1 ^ (r & 7)) << 4)) = zero;
-    for (int b = 0; b < 2; ++b)
-      for (int c = 1; c < 4; c += 2)
-        *reinterpret_cast<uint4*>(smem + C::OFF_COL + b * BLK + r * 128 + ((c ^ (r & 7)) << 4)) = zero;
-    fence_proxy_async_smem();
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -237,24 +220,21 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       // ------------------------------------------------------- S and dA issuer
       constexpr uint32_t idPT = idesc_bf16(128, HT, 0, 0);  // [proto x 64 tokens], K = d, A from TMEM
       const uint64_t dKk = sdesc(sK, 16, 1024), dVk = sdesc(sV, 16, 1024);
-      const uint64_t dCk = sdesc(sbase + C::OFF_COL, 16, 1024), dOne = sdesc(sbase + C::OFF_ONE, 16, 1024);
       auto kstep = [](int k) { return uint32_t((k >> 2) * BLK + (k & 3) * 32); };
       int rc = 0, gc = 0;
       uint32_t fl = info_flags(0);
       for (int li = 0; li < ntiles && ok; ++li) {
         const int ks = li % C::NK, vs = li % C::NV;
-        const uint32_t ofs = uint32_t(li & 1) * BLK;  // per-token operands of this tile
         if (fl & kRunFirst) wt(q_full, uint32_t(rc++) & 1u, 0xD02);
         if (fl & kSegFirst) wt(g_full, uint32_t(gc++) & 1u, 0xD05);
         // everything the first half needs, and the next tile's info, in one round trip
         {
           const uint32_t pp = uint32_t(li - 1) & 1u;  // before the first tile: the phase that counts as done
           const int ln = li + 1 < ntiles ? li + 1 : li;
-          const BarPhase b[5] = {{k_full + 8u * ks, uint32_t(li / C::NK) & 1u},
+          const BarPhase b[4] = {{k_full + 8u * ks, uint32_t(li / C::NK) & 1u},
                                  {v_full + 8u * vs, uint32_t(li / C::NV) & 1u},
                                  {buf_free, pp},
-                                 {i_full + 8u * i_slot(ln), i_par(ln)},
-                                 {TW ? buf_free : col_full + 8u * (li & 1), TW ? pp : uint32_t(li >> 1) & 1u}};
+                                 {i_full + 8u * i_slot(ln), i_par(ln)}};
           ok = ok && mbar_wait_warp_all(b, abort_flag, a.ws, 0xD03);
         }
         if (!ok) break;
@@ -270,22 +250,18 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
           if (elect_one()) {
             const uint64_t dK_ = sdesc_add(dKk, uint32_t(ks) * C::TILE + uint32_t(hf) * (HT * 128));
             const uint64_t dV_ = sdesc_add(dVk, uint32_t(vs) * C::TILE + uint32_t(hf) * (HT * 128));
-            const uint64_t dC_ = sdesc_add(dCk, ofs + uint32_t(hf) * (HT * 128));
-            if (!TW) umma_ss(col + C::S_COL, dOne, dC_, idPT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k)
               umma_ts(col + C::S_COL, tmem + C::Q_COL + 8 * k, sdesc_add(dK_, kstep(k)), idPT,
-                      (!TW || k > 0) ? 1u : 0u);
+                      k > 0 ? 1u : 0u);
             umma_commit(s_full + 8u * hf);
-            if (!TW) umma_ss(col + C::DA_COL, dOne, sdesc_add(dC_, 32u), idPT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k)
               umma_ts(col + C::DA_COL, tmem + C::G_COL + 8 * k, sdesc_add(dV_, kstep(k)), idPT,
-                      (!TW || k > 0) ? 1u : 0u);
+                      k > 0 ? 1u : 0u);
             umma_commit(da_full + 8u * hf);
             if (hf == 1) {
               umma_commit(v_empty + 8u * vs);
-              if (!TW) umma_commit(col_empty + 8u * (li & 1));
               if (fl & kRunLast) umma_commit(q_empty);  // last S of this row of Q
               if (fl & kSegLast) umma_commit(g_empty);  // last dA of this segment
               mbar_arrive(i_empty + 8u * i_slot(li));
@@ -340,16 +316,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       if (elect_one()) umma_commit(drain + 8u);
       mbar_wait_bounded(drain + 8u, 0, 200000000ull);
     } else if (warp == 3 && !TW) {
-      // ------------------------------------------------ per-token operands
-      // x as three bf16 terms (hi, mid, lo) that sum to it; infinities and NaN stay in hi
-      auto split = [](float x) {
-        const float hi = __bfloat162float(__float2bfloat16_rn(x));
-        const float r = x - hi;
-        const float mid = __bfloat162float(__float2bfloat16_rn(r));
-        const bool fin = fabsf(x) < INFINITY && fabsf(hi) < INFINITY;
-        return make_uint4(pack_bf16(hi, fin ? mid : 0.f), pack_bf16(fin ? r - mid : 0.f, 0.f), 0u, 0u);
-      };
-      const float inv = 1.f / (tiny_scale(a.scale) * kLog2e);
+      // ------------------------------------------------ per-token values
       for (int li = 0; li < ntiles && ok; ++li) {
         const int buf = li & 1, ks = li % C::NK;
         wt(i_full + 8u * i_slot(li), i_par(li), 0xE01);
@@ -367,14 +334,12 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
         }
         if (li >= 2) wt(col_empty + 8u * buf, uint32_t((li >> 1) - 1) & 1u, 0xE02);
         if (!ok) break;
-        uint8_t* cl = smem + C::OFF_COL + buf * BLK;
+        float* cl = reinterpret_cast<float*>(smem + C::OFF_COL + buf * C::COL);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int t = lane + 32 * k;
-          *reinterpret_cast<uint4*>(cl + t * 128 + ((0 ^ (t & 7)) << 4)) = split(-x[k].x * inv);
-          *reinterpret_cast<uint4*>(cl + t * 128 + ((2 ^ (t & 7)) << 4)) = split(-x[k].y);
+          cl[lane + 32 * k] = x[k].x;
+          cl[T + lane + 32 * k] = x[k].y;
         }
-        fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(col_full + 8u * buf);
@@ -389,8 +354,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
     const int hf = (warp - kSoftWarp0) >> 2, q = warp & 3;
     const uint32_t lane_off = uint32_t(32 * q) << 16;
     const uint32_t t_half = tmem + lane_off + uint32_t(hf * C::HALF_COLS);
-    const float c2 = (TW ? a.scale : tiny_scale(a.scale)) * kLog2e;
-    const bool no_scores = !TW && a.scale < kTinyScale;
+    const float c2 = a.scale * kLog2e;
     bool ok = true;
     int gc = 0, rc = 0;
     auto wwait = [&](uint32_t bar, uint32_t par, uint32_t site) {
@@ -427,7 +391,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       uint32_t pk[D / 4];
 #pragma unroll
       for (int j = 0; j < D / 16; ++j) {
-        const uint4 x = no_scores ? make_uint4(0u, 0u, 0u, 0u) : src[j];
+        const uint4 x = src[j];
         pk[4 * j] = x.x;
         pk[4 * j + 1] = x.y;
         pk[4 * j + 2] = x.z;
@@ -456,6 +420,15 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
         dr = Dco[r];
       }
       const int left = o.n - HT * hf;  // tokens of this half
+      // the values of 4 tokens a load, ahead of the waits that they would prolong
+      const float4* cl = reinterpret_cast<const float4*>(smem + C::OFF_COL + (li & 1) * C::COL) + (HT / 4) * hf;
+      float4 l4[TW ? 1 : HT / 4];
+      if (!TW) {
+        ok = wwait(col_full + 8u * (li & 1), uint32_t(li >> 1) & 1u, 0xF02);
+        if (!ok) break;
+#pragma unroll
+        for (int j = 0; j < HT / 4; ++j) l4[TW ? 0 : j] = cl[j];
+      }
       ok = wwait(s_full + 8u * hf, uint32_t(li) & 1u, 0xF03);
       if (!ok) break;
       tc_fence_after();
@@ -464,22 +437,42 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
       tmem_ld32(t_half + C::S_COL + 32, sv + 32);
       tmem_ld_wait();
 #pragma unroll
-      for (int j = 0; j < HT; ++j) {
-        if (TW) sv[j] = j < left ? ex2(fmaf(sv[j], c2, -l2r)) : 0.f;
-        else sv[j] = ex2(sv[j] * c2);
+      for (int j = 0; j < HT; j += 4) {
+        if (TW) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) sv[j + i] = j + i < left ? ex2(fmaf(sv[j + i], c2, -l2r)) : 0.f;
+        } else {
+          const float4 l = l4[TW ? 0 : j / 4];
+          sv[j] = ex2(fmaf(sv[j], c2, -l.x));
+          sv[j + 1] = ex2(fmaf(sv[j + 1], c2, -l.y));
+          sv[j + 2] = ex2(fmaf(sv[j + 2], c2, -l.z));
+          sv[j + 3] = ex2(fmaf(sv[j + 3], c2, -l.w));
+        }
+      }
+      float4 d4[TW ? 1 : HT / 4];
+      if (!TW) {
+#pragma unroll
+        for (int j = 0; j < HT / 4; ++j) d4[TW ? 0 : j] = cl[T / 4 + j];
       }
       ok = wwait(da_full + 8u * hf, uint32_t(li) & 1u, 0xF04);
       if (!ok) break;
       tc_fence_after();
-      float dv[HT];
-      tmem_ld32(t_half + C::DA_COL, dv);
-      tmem_ld32(t_half + C::DA_COL + 32, dv + 32);
-      tmem_ld_wait();
       uint32_t pk[HT / 2];
 #pragma unroll
-      for (int j = 0; j < HT / 2; ++j) {
-        if (TW) pk[j] = pack_bf16(sv[2 * j] * (dv[2 * j] - dr), sv[2 * j + 1] * (dv[2 * j + 1] - dr));
-        else pk[j] = pack_bf16(sv[2 * j] * dv[2 * j], sv[2 * j + 1] * dv[2 * j + 1]);
+      for (int c = 0; c < HT; c += 32) {
+        float dv[32];
+        tmem_ld32(t_half + C::DA_COL + c, dv);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          const float4 d = TW ? make_float4(dr, dr, dr, dr) : d4[TW ? 0 : (c + j) / 4];
+          pk[(c + j) / 2] = pack_bf16(sv[c + j] * (dv[j] - d.x), sv[c + j + 1] * (dv[j + 1] - d.y));
+          pk[(c + j) / 2 + 1] = pack_bf16(sv[c + j + 2] * (dv[j + 2] - d.z), sv[c + j + 3] * (dv[j + 3] - d.w));
+        }
+      }
+      if (!TW) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(col_empty + 8u * (li & 1));
       }
       tmem_st16(t_half + C::S_COL, pk);
       tmem_st16(t_half + C::S_COL + 16, pk + 16);
