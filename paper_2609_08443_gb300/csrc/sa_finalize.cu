@@ -12,8 +12,11 @@
 // list), and the list's (segment, column range) items are dealt to all blocks.  Segments of up to
 // kFewPieces pieces (a long batch) give each thread one column and its pieces
 // in order; longer chains (a short batch) are split over the block's eight
-// warps, whose sums are added in warp order.  Both orders depend only on the
-// plan, so the result stays bitwise reproducible.  Measured per call, before and
+// warps, whose sums are added in warp order.  Token-wise segments have [P][d] columns
+// enough for the chip at any length, and their lse and sketch feed the backward's
+// differences, where another order of the sums shows as flipped bf16 roundings: they
+// are always added in piece order, relative to the largest shift.  All orders depend
+// only on the plan, so the result stays bitwise reproducible.  Measured per call, before and
 // after: one user of 1531 tokens 69.6 -> 32.0 us, one fp32 user of 4096 tokens
 // 226 -> 65.6 us, the token-wise step of 12 users (P = 512, d = 128, 215K
 // tokens) 2.99 -> 2.05 ms.
@@ -74,15 +77,13 @@ __device__ __forceinline__ int holder(const int64_t* rb, int W, int64_t t) {
   return lo;
 }
 
-// Running sum of pieces.  Token-wise pieces carry a shift m and a weight sum l
-// (l < 0: no piece); the sum is relative to the largest shift so far, like an
-// online softmax.
+// Sum of pieces.  Token-wise pieces carry a shift m and a weight sum l (l < 0: no
+// piece); the sum is relative to M, the largest shift of the segment.
 template <int V, int KIND>
 struct Acc {
   Col<V> s;
   float M, L;
-  bool any;
-  __device__ __forceinline__ Acc() : M(-INFINITY), L(0.f), any(false) {
+  __device__ __forceinline__ Acc() : M(-INFINITY), L(0.f) {
 #pragma unroll
     for (int k = 0; k < V; ++k) s.x[k] = 0.f;
   }
@@ -93,13 +94,10 @@ struct Acc {
       return;
     }
     if (l < 0.f) return;
-    any = true;
-    const float Mn = fmaxf(M, m);
-    const float fo = expf(M - Mn), fn = expf(m - Mn);
-    L = fmaf(l, fn, L * fo);
+    const float f = expf(m - M);
+    L = fmaf(l, f, L);
 #pragma unroll
-    for (int k = 0; k < V; ++k) s.x[k] = fmaf(v.x[k], fn, s.x[k] * fo);
-    M = Mn;
+    for (int k = 0; k < V; ++k) s.x[k] = fmaf(v.x[k], f, s.x[k]);
   }
 };
 
@@ -108,7 +106,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
   __shared__ int64_t rb[kMaxWorkers + 1];
   __shared__ Seg segs[kMaxWorkers];
   __shared__ int nitems_s;
-  __shared__ float red[kFinWarps][32][V + (KIND == kTokenwise ? 2 : 0)];
+  __shared__ float red[kFinWarps][32][V];
   if (ws_failed(a.ws)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t tph = reinterpret_cast<const WsHeader*>(a.ws)->tiles_per_head;
@@ -154,13 +152,14 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
   }
   __syncthreads();
   const int nseg = KIND == kHeadDq ? a.H : W;
+  auto in_order = [](const Seg& g) { return KIND == kTokenwise || g.g1 - g.g0 < kFewPieces; };
   const int cols = int(PD / V);
   if (warp == 0) {  // exclusive scan of the items per segment
     int carry = 0;
     for (int s = 0; s < nseg; s += 32) {
       int n = 0;
       if (s + lane < nseg && segs[s + lane].row >= 0) {
-        const int per = segs[s + lane].g1 - segs[s + lane].g0 < kFewPieces ? kFinThreads : 32;
+        const int per = in_order(segs[s + lane]) ? kFinThreads : 32;
         n = (cols + per - 1) / per;
       }
       int x = n;
@@ -183,7 +182,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
       if (segs[mid].item0 <= it) lo = mid; else hi = mid - 1;
     }
     const Seg sg = segs[lo];
-    const bool few = sg.g1 - sg.g0 < kFewPieces;
+    const bool few = in_order(sg);
     const int col = (it - sg.item0) * (few ? kFinThreads : 32) + (few ? tid : lane);
     const bool in = col < cols;
     const int64_t e = int64_t(col) * V;
@@ -193,12 +192,18 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
       return KIND == kHeadDq ? int64_t(g) * a.H + sg.row : int64_t(g) * 2 + (rb[g] >= sg.seg0 ? 0 : 1);
     };
     Acc<V, KIND> acc;
-    auto run = [&](int ga, int gb) {  // pieces [ga, gb), four loads in flight
-      for (int g = ga; g < gb; g += 4) {
-        Col<V> v[4];
-        float2 st[4];
+    if (KIND == kTokenwise && in) {
+#pragma unroll 8
+      for (int g = sg.g0; g <= sg.g1; ++g)
+        if (rb[g] != rb[g + 1]) acc.M = fmaxf(acc.M, a.stat[piece(g) * a.P + j].x);
+    }
+    constexpr int U = KIND == kTokenwise ? 8 : 4;
+    auto run = [&](int ga, int gb) {  // pieces [ga, gb), U loads in flight
+      for (int g = ga; g < gb; g += U) {
+        Col<V> v[U];
+        float2 st[U];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < U; ++k) {
           const bool have = in && g + k < gb && rb[g + k] != rb[g + k + 1];
 #pragma unroll
           for (int q = 0; q < V; ++q) v[k].x[q] = 0.f;
@@ -210,7 +215,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
           }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc.add(v[k], st[k].x, st[k].y);
+        for (int k = 0; k < U; ++k) acc.add(v[k], st[k].x, st[k].y);
       }
     };
     auto write = [&]() {
@@ -232,10 +237,6 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
     run(ga, min(ga + per, sg.g1 + 1));
 #pragma unroll
     for (int k = 0; k < V; ++k) red[warp][lane][k] = acc.s.x[k];
-    if (KIND == kTokenwise) {
-      red[warp][lane][V] = acc.M;
-      red[warp][lane][V + 1] = acc.any ? acc.L : -1.f;
-    }
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
         Col<V> v;
 #pragma unroll
         for (int k = 0; k < V; ++k) v.x[k] = red[w][lane][k];
-        acc.add(v, KIND == kTokenwise ? red[w][lane][V] : 0.f, KIND == kTokenwise ? red[w][lane][V + 1] : 0.f);
+        acc.add(v, 0.f, 0.f);
       }
       write();
     }
