@@ -136,6 +136,23 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   return true;
 }
 
+// 32 consecutive floats of one row.  The 32 threads of a warp write 32 different
+// rows, so an instruction touches 32 lines whatever its width: 32-byte stores, which
+// need their alignment, take half as many as 16-byte ones.
+__device__ __forceinline__ void store_row32(float* dst, const float* v) {
+  if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < 32; k += 8)
+      asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + k), "f"(v[k]), "f"(v[k + 1]),
+                   "f"(v[k + 2]), "f"(v[k + 3]), "f"(v[k + 4]), "f"(v[k + 5]), "f"(v[k + 6]), "f"(v[k + 7])
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int k = 0; k < 32; k += 4)
+      *reinterpret_cast<float4*>(dst + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+  }
+}
+
 // Sketch block (PS prototypes x D) from TMEM to global memory.
 //  TRANS (D = 128): TMEM holds O^T: lane = feature d, column = prototype.
 //  else (D = 64):   TMEM holds O in PS/128 blocks: lane = prototype, column = d.
@@ -163,9 +180,7 @@ __device__ __forceinline__ void store_sketch(uint32_t tmem, uint32_t lane_off, i
     for (int c = c0; c < c1; c += 32) {
       ptx::tmem_ld32(tmem + lane_off + O_COL + blk * D + c, v);
       ptx::tmem_ld_wait();
-      float4* o = reinterpret_cast<float4*>(dst + int64_t(p) * D + c);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+      store_row32(dst + int64_t(p) * D + c, v);
     }
   }
 }
@@ -185,10 +200,9 @@ __device__ __forceinline__ void store_sketch_scaled(uint32_t tmem, uint32_t lane
   for (int c = c0; c < c1; c += 32) {
     ptx::tmem_ld32(tmem + lane_off + O_COL + blk * D + c, v);
     ptx::tmem_ld_wait();
-    float4* o = reinterpret_cast<float4*>(dst + int64_t(p) * D + c);
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      o[k] = make_float4(v[4 * k] * mul, v[4 * k + 1] * mul, v[4 * k + 2] * mul, v[4 * k + 3] * mul);
+    for (int k = 0; k < 32; ++k) v[k] *= mul;
+    store_row32(dst + int64_t(p) * D + c, v);
   }
 }
 

@@ -100,9 +100,7 @@ __device__ __forceinline__ void store_block(uint32_t tmem, uint32_t lane_off, in
     const int p = 128 * blk + 32 * q + lane;
     tmem_ld32(tmem + lane_off + C::O_COL + blk * D + c, v);
     tmem_ld_wait();
-    float4* o = reinterpret_cast<float4*>(dst + int64_t(p) * D + c);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    store_row32(dst + int64_t(p) * D + c, v);
   }
 }
 
