@@ -6,7 +6,7 @@
 // computed first (simt_lse_kernel), then blocks of 64 prototypes accumulate
 // A[j,i] V_i with A[j,i] = exp(S[j,i] - lse_i) over a worker's tile range.
 // Backward (chain rule of Sec. 3.1): per token tile dV and D_i = dV_i . v_i,
-// then dK; dQ is accumulated per worker and head and reduced in worker order.
+// then dK; dQ is accumulated per worker and head and reduced in a fixed order.
 #include <type_traits>
 
 #include "sa_kernels.cuh"

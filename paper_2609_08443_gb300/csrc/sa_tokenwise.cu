@@ -17,7 +17,7 @@
 //     dK_i = scale sum_j dS[j,i] q_j,    dQ[h] = scale sum_b sum_i dS[:, i] k_i.
 // D_j depends only on the forward's output, so the token side (dV, dK) needs a
 // single pass over the prototypes; dQ is accumulated per worker and head and
-// reduced in worker order by the shared finalize kernel.
+// reduced in a fixed order by the shared finalize kernel.
 //
 // CUDA cores, fp32 arithmetic, inputs fp32 or bf16 (widened on load).
 #include "sa_simt_util.cuh"

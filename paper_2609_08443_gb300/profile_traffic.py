@@ -65,7 +65,8 @@ def main():
         res[name] = {"bytes_per_launch": e["bytes"] / e["launches"] * scale, "captured_launches": e["launches"],
                      "scale": scale, "source_hash": h}
     # the backward's two main kernels count as one call, as the bench times them
-    for tok_pre, dq_pre in (("tc_bwd_tok_kernel", "tc_bwd_dq_kernel"), ("tc_tw_bwd_tok_kernel", "tc_tw_bwd_dq_kernel")):
+    for tok_pre, dq_pre in (("tc_bwd2_kernel", "tc_bwd_dq_kernel"), ("tc_bwd_tok_kernel", "tc_bwd_dq_kernel"),
+                            ("tc_tw_bwd_tok_kernel", "tc_tw_bwd_dq_kernel")):
         tok = next((k for k in res if k.startswith(tok_pre)), None)
         dq = next((k for k in res if k.startswith(dq_pre)), None)
         if tok and dq:
