@@ -64,6 +64,10 @@ def main():
     for name, e in sorted(agg.items()):
         res[name] = {"bytes_per_launch": e["bytes"] / e["launches"] * scale, "captured_launches": e["launches"],
                      "scale": scale, "source_hash": h}
+    # the two-sweep backward's names as the library gives them: <d,P> or, dQ fused, <d,P,dq>
+    for name in [k for k in res if k.startswith("tc_bwd2_kernel")]:
+        d, p, fuse = name[len("tc_bwd2_kernel<"):-1].split(",")[:3]
+        res[f"tc_bwd2_kernel<{d},{p}{',dq' if fuse in ('1', 'true') else ''}>"] = res.pop(name)
     # the backward's two main kernels count as one call, as the bench times them
     for tok_pre, dq_pre in (("tc_bwd2_kernel", "tc_bwd_dq_kernel"), ("tc_bwd_tok_kernel", "tc_bwd_dq_kernel"),
                             ("tc_tw_bwd_tok_kernel", "tc_tw_bwd_dq_kernel")):
