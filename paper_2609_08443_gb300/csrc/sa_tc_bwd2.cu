@@ -40,6 +40,7 @@
 // own queries 0.61 and 0.54 ms.
 #include <cuda.h>
 
+#include "sa_handoff.cuh"
 #include "sa_ptx.cuh"
 #include "sa_tc.cuh"
 #include "sa_tc_common.cuh"
@@ -73,8 +74,7 @@ struct SCfg {
   static constexpr bool Q_RES = !(D == 128 && P == 512);
   static constexpr int NQ = Q_RES ? NCH * ND : 2;  // Q blocks in shared memory
   // Q barriers: one, or when streamed two slots whose blocks announce themselves on
-  // eight barriers in turn.  The two issuers each see only their own blocks, at
-  // most eight apart, so a parity never stands for the wrong block.
+  // eight barriers in turn (sa_handoff.cuh)
   static constexpr int NQF = Q_RES ? 1 : 8, NQE = Q_RES ? 1 : 2;
   static_assert(Q_RES || (NCH == 4 && ND == 2), "streamed blocks of one issuer are at most eight apart");
   static constexpr int NG = FUSE && D == 64 ? 2 : 1;  // G buffers (the next user's is converted meanwhile)
@@ -91,7 +91,8 @@ struct SCfg {
   static constexpr bool SPLIT_D = D == 128;  // D_i from two half dots, exchanged between the warpgroups
   static constexpr int OFF_INFO = OFF_STATS + (SPLIT_D ? 2 * 2 * T * 4 : 0);
   static constexpr int OFF_BAR = OFF_INFO + NI * int(sizeof(TileInfo));
-  static constexpr int NBAR = 2 * NK + 2 * NV + NQF + NQE + 2 * NGB + 2 * NI + NCH + 12;
+  static constexpr int NCB = handoff::chunk_bars(NCH);
+  static constexpr int NBAR = 2 * NK + 2 * NV + NQF + NQE + 2 * NGB + 2 * NI + NCH + 2 * NCB + 8;
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
   static constexpr int SMEM = OFF_MISC + 16;
   static constexpr int SD_COL = 0, A_COL = NC, DV_COL = A_COL + P / 2;
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t k_full = take(C::NK), k_empty = take(C::NK), v_full = take(C::NV), v_empty = take(C::NV),
                  q_full = take(C::NQF), q_empty = take(C::NQE), g_full = take(C::NGB), g_empty = take(C::NGB),
                  i_full = take(C::NI), i_empty = take(C::NI), dk_done = take(NCH), sd_full = take(1),
-                 sd_free = take(1), a_full = take(2), dv_full = take(1), ds_full = take(2), acc_free = take(1),
+                 sd_free = take(1), a_full = take(C::NCB), dv_full = take(1), ds_full = take(C::NCB), acc_free = take(1),
                  dq_free = take(1), st_ready = take(1), drain = take(2);
   TileInfo* infos = reinterpret_cast<TileInfo*>(smem + C::OFF_INFO);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
@@ -193,9 +194,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     init(dk_done, NCH, 1);
     init(sd_full, 1, 1);
     init(sd_free, 1, kSoftWarps);
-    init(a_full, 2, kSoftWarps);
+    init(a_full, C::NCB, kSoftWarps);
     init(dv_full, 1, 1);
-    init(ds_full, 2, kSoftWarps);
+    init(ds_full, C::NCB, kSoftWarps);
     init(acc_free, 1, kSoftWarps);
     init(dq_free, 1, kSoftWarps);
     init(st_ready, 1, kSoftWarps);
@@ -210,11 +211,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = *tmem_slot;
   auto i_slot = [](int li) { return li % C::NI; };
   auto i_par = [](int li) { return uint32_t(li / C::NI) & 1u; };
-  // a_full and ds_full alternate between two barriers from chunk to chunk: a warp
-  // may arrive for the next chunk before a slower one has for this, and for the
-  // one after only once every warp has freed S/dA of the next, past this arrival
-  auto chunk_bar = [](int li, int c) { return 8u * (uint32_t(li * NCH + c) & 1u); };
-  auto chunk_par = [](int li, int c) { return (uint32_t(li * NCH + c) >> 1) & 1u; };
+  auto chunk_bar = [](int li, int c) { return 8u * uint32_t(handoff::chunk_bar(li, c, NCH)); };
+  auto chunk_par = [](int li, int c) { return handoff::chunk_parity(li, c, NCH); };
 
   if (ntiles > 0 && warp < kSoftWarp0) {
     setmaxnreg_dec<kRegsCtl>();
@@ -316,17 +314,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       auto g_ofs = [&](int c) { return uint32_t((FUSE ? int(gseg % C::NG) * NCH : 0) + c) * uint32_t(C::TILE); };
       auto g_bar = [&](int c) { return g_empty + 8u * (FUSE ? int(gseg % C::NG) : c); };
-      // streamed Q blocks are consumed in the loader's order: S_0(0); per tile S_1 ..,
-      // dK_0 .. dK_(last-1), S_0 of the next tile, dK_last
-      constexpr uint32_t kPerTile = 2 * NCH * ND;
-      auto qb_S = [&](int li, int c) -> uint32_t {
-        if (c > 0) return ND + uint32_t(li) * kPerTile + uint32_t(c - 1) * ND;
-        return li > 0 ? ND + uint32_t(li - 1) * kPerTile + 2u * (NCH - 1) * ND : 0u;
-      };
-      auto qb_dK = [&](int li, int c) -> uint32_t {
-        const uint32_t base = ND + uint32_t(li) * kPerTile;
-        if (c + 1 < NCH) return base + uint32_t(NCH - 1 + c) * ND;
-        return base + 2u * (NCH - 1) * ND + (li + 1 < ntiles ? ND : 0u);
+      auto qb_S = [&](int li, int c) { return handoff::q_block_of_S(li, c, NCH, ND); };
+      auto qb_dK = [&](int li, int c) { return handoff::q_block_of_dK(li, c, li + 1 >= ntiles, NCH, ND); };
+      auto q_phase = [&](uint32_t x) {
+        return BarPhase{q_full + 8u * handoff::q_block_bar(x), handoff::q_block_parity(x)};
       };
       if (warp == 1) {
         constexpr uint32_t idS = idesc_bf16(128, C::NC, 0, 0);  // [tok x chunk], K = d
@@ -359,12 +350,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           } else {
             const uint32_t qb = qb_S(li, c);
-            const BarPhase b[3] = {kf, sd_phase(kf), {q_full + 8u * (qb & 7u), (qb >> 3) & 1u}};
+            const BarPhase b[3] = {kf, sd_phase(kf), q_phase(qb)};
             ok = ok && mbar_wait_warp_all(b, abort_flag, a.ws, 0xD15);
 #pragma unroll
             for (int dh = 0; dh < ND; ++dh) {
               const uint32_t x = qb + uint32_t(dh), s = x & 1u;
-              if (dh > 0) wt(q_full + 8u * (x & 7u), (x >> 3) & 1u, 0xD16);
+              if (dh > 0) wt(q_phase(x).bar, q_phase(x).parity, 0xD16);
               if (!ok) return;
               tc_fence_after();
               if (elect_one()) {
@@ -468,12 +459,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           } else {
             const uint32_t qb = qb_dK(li, c);
-            const BarPhase b[3] = {df, af, {q_full + 8u * (qb & 7u), (qb >> 3) & 1u}};
+            const BarPhase b[3] = {df, af, q_phase(qb)};
             ok = ok && mbar_wait_warp_all(b, abort_flag, a.ws, 0xD1B);
 #pragma unroll
             for (int dh = 0; dh < ND; ++dh) {
               const uint32_t x = qb + uint32_t(dh), s = x & 1u;
-              if (dh > 0) wt(q_full + 8u * (x & 7u), (x >> 3) & 1u, 0xD1E);
+              if (dh > 0) wt(q_phase(x).bar, q_phase(x).parity, 0xD1E);
               if (!ok) return;
               tc_fence_after();
               if (elect_one()) {
@@ -588,8 +579,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t s = qb & 1u;
           if (qb >= 2u) ok = ok && mbar_wait(q_empty + 8u * s, ((qb >> 1) + 1) & 1u, abort_flag, a.ws, 0xE14);
           if (!ok) return;
-          mbar_arrive_expect_tx(q_full + 8u * (qb & 7u), BLK);
-          tma_load_3d(sQ + s * BLK, &tmQ, q_full + 8u * (qb & 7u), 64 * dh, c * C::NC, qk);
+          const uint32_t full = q_full + 8u * handoff::q_block_bar(qb);
+          mbar_arrive_expect_tx(full, BLK);
+          tma_load_3d(sQ + s * BLK, &tmQ, full, 64 * dh, c * C::NC, qk);
         }
       };
       int qk = 0, row = 0;
@@ -626,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) {  // the copies in flight land before the CTA may exit
         for (uint32_t k = qb > 2u ? qb - 2u : 0u; k < qb; ++k)
-          mbar_wait_bounded(q_full + 8u * (k & 7u), (k >> 3) & 1u, 200000000ull);
+          mbar_wait_bounded(q_full + 8u * handoff::q_block_bar(k), handoff::q_block_parity(k), 200000000ull);
         for (int c = 0; c < NCH; ++c) {
           const int n = gc + (c < loaded_g ? 1 : 0);  // loads of chunk c so far
           if (n > 0) mbar_wait_bounded(g_full + 8u * c, uint32_t(n - 1) & 1u, 200000000ull);
