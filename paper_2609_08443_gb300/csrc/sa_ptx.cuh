@@ -102,7 +102,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 
 // Several barriers at once.  A shared-memory access takes 250-400 cycles beside
 // running tensor-core products, so the polls are issued back to back and their
-// latencies overlap; only what is not complete yet is then waited for in turn.
+// latencies overlap.  If one is not complete yet they are all waited for in turn, also
+// those that the first round saw: no barrier named here completes its next phase before
+// this warp is past the wait, so a phase that was seen still reads as complete.  (Asking
+// only for the rest cost more instructions than the repeated polls: step of 16 users of
+// 100K tokens, P = 512, d = 128, 13.00 and 13.18 ms; rounds of joined polls 13.45 ms.)
 struct BarPhase {
   uint32_t bar, parity;
 };
