@@ -130,11 +130,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
   using C = TokCfg<D, P>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  if (ws_failed(a.ws)) return;
-  if (smem_u32(smem) & 1023u) {
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB21u);
-    return;
-  }
+  if (cta_leaves(a.ws, smem_u32(smem), 0xB21u)) return;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t sSlots = sbase + C::OFF_SLOTS, sAB = sbase + C::OFF_AB;
   auto slot_addr = [&](int s) { return sSlots + uint32_t(s) * C::SLOT; };

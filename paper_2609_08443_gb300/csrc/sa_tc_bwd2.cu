@@ -148,11 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int NCH = C::NCH, ND = C::ND, BLK = C::BLK;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  if (ws_failed(a.ws)) return;
-  if (smem_u32(smem) & 1023u) {  // 128-byte swizzle atoms need 1024-byte alignment
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB41u);
-    return;
-  }
+  if (cta_leaves(a.ws, smem_u32(smem), 0xB41u)) return;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t sG = sbase + C::OFF_G, sQ = sbase + C::OFF_Q, sK = sbase + C::OFF_K, sV = sbase + C::OFF_V,
                  sDS = sbase + C::OFF_DS;

@@ -92,13 +92,7 @@ __device__ __forceinline__ void bwd_dq_body(const CUtensorMap& tmK, const CUtens
   constexpr int ND = C::ND, BLK = C::BLK, HT = C::HT;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  // early exits by vote: after one that could split a warp, nothing below would be
-  // compiled as warp-uniform (uniform registers and branches of the issuing warps)
-  if (__any_sync(0xffffffffu, ws_failed(a.ws))) return;
-  if (smem_u32(smem) & 1023u) {
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xB31u);
-    return;
-  }
+  if (cta_leaves(a.ws, smem_u32(smem), 0xB31u)) return;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t sK = sbase + C::OFF_K, sV = sbase + C::OFF_V, sRaw = sbase + C::OFF_RAW;
   const float2* tokv = reinterpret_cast<const float2*>(Dco);  // prototype-wise: [H][N]

@@ -116,6 +116,17 @@ struct TileWalkerSearch : TileWalker {
   }
 };
 
+// Whether this CTA leaves before any set-up: the call has failed, or the base is not on
+// the 1024 bytes that the 128-byte swizzle atoms need (recorded under `site`).  Another CTA
+// of the same launch may set the error word, when a wait gives up, between two threads'
+// reads of it, so the CTA votes: all of its threads leave or none, and no warp runs on
+// without the barriers and the tensor memory that another one was to set up.
+__device__ __forceinline__ bool cta_leaves(void* ws, uint32_t smem_base, uint32_t site) {
+  const bool misaligned = (smem_base & 1023u) != 0u;
+  if (misaligned && threadIdx.x == 0) ws_set_error(ws, SA_ERR_CUDA, site);
+  return __syncthreads_or(misaligned || ws_failed(ws)) != 0;
+}
+
 // Where a worker's dQ block of prototypes [p0, p0 + PS) for the tiles ending
 // at walker position w goes.  Shared queries: the worker's partial of head h
 // ([W][H][P][d], summed over workers afterwards).  Per-user queries: dQ[b, h]

@@ -114,11 +114,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // Both CTAs of a pair must reach the cluster barriers below, so a failed
   // call or a misaligned base only skips the work.
-  bool skip = ws_failed(a.ws);
-  if (smem_u32(smem) & 1023u) {
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xA31u);
-    skip = true;
-  }
+  const bool skip = cta_leaves(a.ws, smem_u32(smem), 0xA31u);
   const uint32_t sbase = smem_u32(smem);
   const uint32_t sQ = sbase + C::OFF_Q, sK = sbase + C::OFF_K, sV = sbase + C::OFF_V, sW = sbase + C::OFF_W;
   const uint32_t bar0 = sbase + C::OFF_BAR;

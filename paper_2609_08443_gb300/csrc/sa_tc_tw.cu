@@ -68,11 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = Cfg<D, NM>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  if (ws_failed(a.ws)) return;
-  if (smem_u32(smem) & 1023u) {  // 128-byte swizzle atoms need 1024-byte alignment
-    if (threadIdx.x == 0) ws_set_error(a.ws, SA_ERR_CUDA, 0xA21u);
-    return;
-  }
+  if (cta_leaves(a.ws, smem_u32(smem), 0xA21u)) return;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t sQ = sbase + C::OFF_Q, sRing = sbase + C::OFF_RING, sW = sbase + C::OFF_W;
   const uint32_t bar0 = sbase + C::OFF_BAR;
