@@ -200,6 +200,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
       auto load = [&](int s, const CUtensorMap* map, int c1, int c2) {
         if ((used >> s) & 1u) {
           ok = ok && mbar_wait(empty_bar(s), (par >> s) & 1u, abort_flag, a.ws, 0x801);
+          if (!ok) return;  // par stays that of the slot's last load, which the drain below waits for
           par ^= 1u << s;
         }
         if (!ok) return;

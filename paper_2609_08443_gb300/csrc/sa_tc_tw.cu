@@ -172,6 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) {  // drain loads still in flight before the CTA may exit
         for (uint32_t k = (e > uint32_t(C::NSLOT) ? e - C::NSLOT : 0); k < e; ++k)
           mbar_wait_bounded(ring_full(int(k % C::NSLOT)), (k / C::NSLOT) & 1, 200000000ull);
+        if (hc > 0) mbar_wait_bounded(q_full, uint32_t(hc - 1) & 1u, 200000000ull);
       }
     } else if (warp == 1) {
       // ------------------------------------------------------ UMMA issuer

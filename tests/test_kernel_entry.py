@@ -69,3 +69,29 @@ def test_failed_call_leaves_and_the_next_is_clean(cuda_lib, P, d, path):
             assert all(torch.equal(x, y) for x, y in zip(out, ref))
     finally:
         binding.sa_select_path(0)
+
+
+def kernels():
+    """(file, text) of each tensor-core kernel from its set-up to its TMEM release."""
+    for path in SOURCES:
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"extern __shared__[^;]*;(.*?)tmem_dealloc\(", text, flags=re.S):
+            yield os.path.basename(path), m.group(1)
+
+
+@pytest.mark.parametrize("where,text", list(kernels()), ids=lambda x: x[:16] if x.endswith(".cu") else "")
+def test_abort_waits_for_every_copy(where, text):
+    """A role that gives up waits for its copies in flight: every barrier that a copy into
+    shared memory completes has its bounded wait (the peer's pushes, x_full and r_full,
+    are no copies of the waiting CTA)."""
+    full = set(re.findall(r"mbar_arrive_expect_tx\((\w+)", text)) - {"x_full", "r_full"}
+    if "full" in full:  # a streamed block's barrier, one of q_full
+        full = full - {"full"} | {"q_full"}
+    assert full, where
+    assert full <= set(re.findall(r"mbar_wait_bounded\((\w+)", text)), where
+
+
+def test_slot_parity_stays_that_of_the_last_load():
+    text = open(os.path.join(build.CSRC, "sa_tc_bwd.cu")).read()
+    load = re.search(r"auto load = .*?used \|= 1u << s;", text, flags=re.S).group(0)
+    assert re.search(r"mbar_wait\(empty_bar\(s\)[^;]*;\s*if \(!ok\) return;[^\n]*\n\s*par \^= 1u << s;", load)
