@@ -23,6 +23,10 @@
  *     besides per-device caches (kernel attributes, SM count, timing events).
  *   - K, V, Q, dK, dV all have element type `dt`.  sketch, dsketch, dQ and lse
  *     are float32.  Element offsets are 64-bit.
+ *   - K, V and Q (X and Wk of the key projection) start on 16-byte boundaries; so
+ *     do dK, dV and dX where the tensor cores serve the backward (bf16, d in {64,
+ *     128}, P in {128, 256, 512, 1024, 2048}; token-wise d = 128 and P >= 256).
+ *     Others are refused with SA_ERR_INVALID_ARG.
  *   - K, V   : [N, H, d]   packed rows of all users, N = cu_seqlens[B]
  *     Q      : [H, P, d]   prototypes
  *     cu     : [B + 1]     int32, cu[0] = 0, non-decreasing, cu[B] = N
@@ -35,8 +39,8 @@
  *   - Inputs and outputs must not overlap.
  *   - Results are bitwise reproducible for the same inputs, device and
  *     arguments: every reduction runs in a fixed order (no float atomics).
- *   - Errors the host can see (NULL pointers, sizes, unsupported shapes, a small
- *     workspace) are returned synchronously before anything is enqueued.
+ *   - Errors the host can see (NULL pointers, sizes, unsupported shapes, misaligned
+ *     buffers, a small workspace) are returned synchronously before anything is enqueued.
  *     Errors only the device can see (bad cu_seqlens contents, a pipeline wait
  *     that gave up) are written to an error word inside the workspace; the
  *     kernels of that call then skip their work, and sa_get_device_error()
@@ -55,7 +59,7 @@ extern "C" {
 
 typedef enum {
   SA_OK = 0,
-  SA_ERR_INVALID_ARG = 1,  /* NULL pointer, negative size, scale not finite     */
+  SA_ERR_INVALID_ARG = 1,  /* NULL or misaligned pointer, bad size or scale     */
   SA_ERR_UNSUPPORTED = 2,  /* shape or dtype outside what the kernels support   */
   SA_ERR_WORKSPACE = 3,    /* ws_bytes smaller than sa_workspace_size()          */
   SA_ERR_CUDA = 4,         /* a CUDA runtime call failed (launch, event, ...)    */

@@ -308,15 +308,26 @@ sa_status fwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
   return SA_OK;
 }
 
+// What the backward's host can see, before anything is enqueued: its kernels for the
+// call in *plan, or the error.
+sa_status bwd_check(const void* K, const void* V, const int32_t* cu_seqlens, int B, int64_t N, const void* Q, int H,
+                    int P, int d, float scale, sa_dtype dt, const float* dsketch, const void* dK, const void* dV,
+                    const float* dQ, const void* workspace, size_t ws_bytes, int uq, Plan* plan) {
+  if (!dsketch || !dQ || (N > 0 && (!dK || !dV))) return SA_ERR_INVALID_ARG;
+  SA_TRY(check_common(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, ws_bytes, true, uq, plan));
+  // 16-byte stores and TMA stores
+  if (plan->bwd_path == Path::TcBwd && N > 0 && (!aligned16(dK) || !aligned16(dV))) return SA_ERR_INVALID_ARG;
+  return SA_OK;
+}
+
 // Backward of both entry points; uq = 1: Q and dQ hold one [H, P, d] block per
 // user, whose pieces from different workers are summed like the sketch's.
-// sum_dx = 1 (shapes with bwd_on_tc): dV receives dV + dK and dK is not written.
+// sum_dx = 1 (tensor-core shapes): dV receives dV + dK and dK is not written.
 sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int B, int64_t N, const void* Q, int H,
                    int P, int d, float scale, sa_dtype dt, const float* dsketch, const float* lse, void* dK,
                    void* dV, float* dQ, void* workspace, size_t ws_bytes, void* stream, int uq, int sum_dx = 0) {
-  if (!dsketch || !dQ || (N > 0 && (!dK || !dV))) return SA_ERR_INVALID_ARG;
   Plan plan;
-  SA_TRY(check_common(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, ws_bytes, true, uq, &plan));
+  SA_TRY(bwd_check(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, dsketch, dK, dV, dQ, workspace, ws_bytes, uq, &plan));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   sa::Args a = make_args(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, plan.lay);
   a.uq = uq;
@@ -446,11 +457,14 @@ sa_status sa_sketch_bwd_x(const void* X, const int32_t* cu_seqlens, int B, int64
   float* dQf = reinterpret_cast<float*>(Qf + sa::align256(size_t(H) * P * d * x_elem(dt)));
   char* dKf = reinterpret_cast<char*>(dQf) + sa::align256(size_t(H) * P * d * 4);
   const bool sum_dx = x_sums_dx(P, d, dt);
+  void* dK = N > 0 ? (sum_dx ? dX : dKf) : nullptr;
+  Plan plan;
+  SA_TRY(bwd_check(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, dsketch, dK, dX, dQf, workspace, base, 0, &plan));
   SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_fold_wk(Q, Wk, H, P, d, dt, Qf, st); }));
   // the step with K = V = X and prototypes Q': dX = dV + dK' from the backward's
   // epilogue, or dV into dX and dK' to the workspace and a pass that adds them
-  SA_TRY(bwd_impl(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, dsketch, lse,
-                  N > 0 ? (sum_dx ? dX : dKf) : nullptr, dX, dQf, workspace, base, stream, 0, sum_dx ? 1 : 0));
+  SA_TRY(bwd_impl(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, dsketch, lse, dK, dX, dQf, workspace, base, stream,
+                  0, sum_dx ? 1 : 0));
   if (!sum_dx)
     SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_add_into(dX, dKf, N * H * int64_t(d), dt, st); }));
   return launch(SA_KERNEL_AUX, st, [&] { return sa::launch_wk_grads(dQf, Q, Wk, H, P, d, dt, dQ, dWk, st); });
@@ -563,6 +577,7 @@ sa_status sa_sketch_bwd_tokenwise(const void* K, const void* V, const int32_t* c
     return SA_ERR_INVALID_ARG;
   TwLayout lay;
   SA_TRY(tw_check(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, ws_bytes, true, &lay));
+  if (lay.tc_bwd && N > 0 && (!aligned16(dK) || !aligned16(dV))) return SA_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(workspace);
   sa::Args a = make_args(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, lay.base);

@@ -105,8 +105,9 @@ struct SCfg {
   static_assert(OFF_INFO % 16 == 0 && OFF_BAR % 8 == 0, "alignment");
 };
 
-// 64 (or 32) bf16 values, 32 packed words at most, to a 16-byte aligned row:
-// 32-byte stores where the row allows them (whole sectors per thread).
+// 64 (or 32) bf16 values, 32 packed words at most, to a 16-byte aligned row (the
+// entry points refuse others): 32-byte stores where the row allows them (whole
+// sectors per thread).
 template <int NW>
 __device__ __forceinline__ void store_packed(__nv_bfloat16* dst, const uint32_t* pk, bool by32) {
   if (by32) {
@@ -842,7 +843,6 @@ static cudaError_t launch_t(const Args& a, int W, const float* dsk, const __nv_b
                             float* Dco, void* dK, void* dV, cudaStream_t st) {
   using C = SCfg<D, P, FUSE, SUM>;
   CUtensorMap tk, tv, tq, tg;
-  if (((reinterpret_cast<uintptr_t>(dK) | reinterpret_cast<uintptr_t>(dV)) & 15) != 0) return cudaErrorInvalidValue;
   if (!make_kv_map(&tk, a.K, a.N, a.H, D) || !make_kv_map(&tv, a.V, a.N, a.H, D) ||
       !make_q_map(&tq, a.Q, a.uq ? a.B * a.H : a.H, a.P, D, C::NC))
     return cudaErrorInvalidValue;

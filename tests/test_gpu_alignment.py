@@ -1,0 +1,72 @@
+"""Buffers off the boundaries that the tensor-core kernels need: refused with
+SA_ERR_INVALID_ARG before anything is enqueued, on every entry point."""
+import pytest
+import torch
+
+from paper_2609_08443_gb300 import binding, workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(256, 64), (128, 128), (512, 64), (512, 128), (1024, 128)]
+
+
+def inputs(P, d, per_user_q=False):
+    spec = wl.custom([300, 33], H=2, P=P, d=d, dtype=wl.BF16, seed=5)
+    return spec, wl.host_to_torch(spec, wl.make_host(spec, per_user_q=per_user_q), torch.device("cuda"))
+
+
+def off(t):
+    """A buffer like t one element past a 16-byte boundary, with its values."""
+    x = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)[1:].view(t.shape)
+    return x.copy_(t)
+
+
+def refused(call):
+    n = binding.sa_launch_count()
+    with pytest.raises(binding.SketchError) as e:
+        call()
+    assert e.value.status == 1
+    assert binding.sa_launch_count() == n
+
+
+def raw(entry, *args):
+    binding._check(entry(*(a.data_ptr() if isinstance(a, torch.Tensor) else a for a in args)), "entry")
+
+
+def stream():
+    return torch.cuda.current_stream().cuda_stream
+
+
+@pytest.mark.parametrize("which", [0, 1], ids=["dK", "dV"])
+@pytest.mark.parametrize("P,d", SHAPES, ids=lambda x: str(x))
+def test_gradient_rows(cuda_lib, P, d, which):
+    spec, t = inputs(P, d)
+    outs = [torch.empty_like(t["K"]), torch.empty_like(t["K"]), torch.empty(t["Q"].shape, device="cuda")]
+    outs[which] = off(outs[which])
+    a = (t["K"], t["V"], t["cu_seqlens"], t["Q"], t["dsketch"], spec.scale)
+    refused(lambda: binding.sa_sketch_bwd(*a, outs=outs))
+
+
+@pytest.mark.parametrize("P,d", SHAPES, ids=lambda x: str(x))
+def test_dx(cuda_lib, P, d):
+    spec, t = inputs(P, d)
+    lib, H = binding.load(), 2
+    Wk = torch.zeros(H, d, d, dtype=torch.bfloat16, device="cuda")
+    N, B = t["K"].shape[0], 2
+    ws = torch.empty(lib.sa_workspace_size_x(B, N, H, P, d, 1, 1), dtype=torch.uint8, device="cuda")
+    dQ, dWk = torch.empty(H, P, d, device="cuda"), torch.empty(H, d, d, device="cuda")
+    refused(lambda: raw(lib.sa_sketch_bwd_x, t["K"], t["cu_seqlens"], B, N, t["Q"], Wk, H, P, d, spec.scale, 1,
+                        t["dsketch"], None, off(t["K"]), dQ, dWk, ws, ws.numel(), stream()))
+
+
+@pytest.mark.parametrize("which", [0, 1], ids=["dK", "dV"])
+def test_tokenwise_gradient_rows(cuda_lib, which):
+    P, d, H = 512, 128, 2
+    spec, t = inputs(P, d)
+    lib, N, B = binding.load(), t["K"].shape[0], 2
+    ws = torch.empty(lib.sa_workspace_size_tokenwise(B, N, H, P, d, 1, 1), dtype=torch.uint8, device="cuda")
+    outs = [torch.empty_like(t["K"]), torch.empty_like(t["K"])]
+    outs[which] = off(outs[which])
+    dQ = torch.empty(H, P, d, device="cuda")
+    refused(lambda: raw(lib.sa_sketch_bwd_tokenwise, t["K"], t["V"], t["cu_seqlens"], B, N, t["Q"], H, P, d,
+                        spec.scale, 1, None, None, t["dsketch"], *outs, dQ, ws, ws.numel(), stream()))
