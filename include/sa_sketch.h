@@ -23,10 +23,11 @@
  *     besides per-device caches (kernel attributes, SM count, timing events).
  *   - K, V, Q, dK, dV all have element type `dt`.  sketch, dsketch, dQ and lse
  *     are float32.  Element offsets are 64-bit.
- *   - K, V and Q (X and Wk of the key projection) start on 16-byte boundaries; so
- *     do dK, dV and dX where the tensor cores serve the backward (bf16, d in {64,
- *     128}, P in {128, 256, 512, 1024, 2048}; token-wise d = 128 and P >= 256).
- *     Others are refused with SA_ERR_INVALID_ARG.
+ *   - K, V and Q (X and Wk of the key projection) start on 16-byte boundaries.
+ *     Where the tensor cores serve the call (bf16, d in {64, 128}, P in {128, 256,
+ *     512, 1024, 2048}; for the token-wise variant see there) so do dK, dV and dX.
+ *     Others are refused with SA_ERR_INVALID_ARG.  The sketch, lse and dQ
+ *     may start on any 4 bytes.
  *   - K, V   : [N, H, d]   packed rows of all users, N = cu_seqlens[B]
  *     Q      : [H, P, d]   prototypes
  *     cu     : [B + 1]     int32, cu[0] = 0, non-decreasing, cu[B] = N

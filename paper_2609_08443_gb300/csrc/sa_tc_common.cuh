@@ -147,9 +147,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   return true;
 }
 
-// 32 consecutive floats of one row.  The 32 threads of a warp write 32 different
-// rows, so an instruction touches 32 lines whatever its width: 32-byte stores, which
-// need their alignment, take half as many as 16-byte ones.  Forward kernel, 1024 short users
+// 32 consecutive floats of one row, which may start on any 4 bytes (the caller's sketch).
+// The 32 threads of a warp write 32 different rows, so an instruction touches 32 lines
+// whatever its width: 32-byte stores, which need their alignment, take half as many as
+// 16-byte ones.  Forward kernel, 1024 short users
 // and one of 1M tokens (P = 256, d = 64): 1.93 ms with 16-byte stores, 1.72 ms with these.
 __device__ __forceinline__ void store_row32(float* dst, const float* v) {
   if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
@@ -158,10 +159,13 @@ __device__ __forceinline__ void store_row32(float* dst, const float* v) {
       asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + k), "f"(v[k]), "f"(v[k + 1]),
                    "f"(v[k + 2]), "f"(v[k + 3]), "f"(v[k + 4]), "f"(v[k + 5]), "f"(v[k + 6]), "f"(v[k + 7])
                    : "memory");
-  } else {
+  } else if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
 #pragma unroll
     for (int k = 0; k < 32; k += 4)
       *reinterpret_cast<float4*>(dst + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) dst[k] = v[k];
   }
 }
 

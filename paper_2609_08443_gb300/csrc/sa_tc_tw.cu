@@ -353,10 +353,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int c = 0; c < D; c += 32) {
             tmem_ld32(tmem + lane_off + C::O_COL + g * D + c, o);
             tmem_ld_wait();
-            float4* d4 = reinterpret_cast<float4*>(dst + c);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              d4[k] = make_float4(o[4 * k] * mul, o[4 * k + 1] * mul, o[4 * k + 2] * mul, o[4 * k + 3] * mul);
+            for (int k = 0; k < 32; ++k) o[k] *= mul;
+            store_row32(dst + c, o);
           }
           if (whole)
             lse_tok[row * a.P + p0 + pr] = msh * kLn2 + logf(l);

@@ -1,5 +1,6 @@
 """Buffers off the boundaries that the tensor-core kernels need: refused with
-SA_ERR_INVALID_ARG before anything is enqueued, on every entry point."""
+SA_ERR_INVALID_ARG before anything is enqueued, on every entry point; outputs that
+need none give the same bits wherever they start."""
 import pytest
 import torch
 
@@ -10,8 +11,8 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(256, 64), (128, 128), (512, 64), (512, 128), (1024, 128)]
 
 
-def inputs(P, d, per_user_q=False):
-    spec = wl.custom([300, 33], H=2, P=P, d=d, dtype=wl.BF16, seed=5)
+def inputs(P, d, per_user_q=False, lens=(300, 33)):
+    spec = wl.custom(list(lens), H=2, P=P, d=d, dtype=wl.BF16, seed=5)
     return spec, wl.host_to_torch(spec, wl.make_host(spec, per_user_q=per_user_q), torch.device("cuda"))
 
 
@@ -70,3 +71,38 @@ def test_tokenwise_gradient_rows(cuda_lib, which):
     dQ = torch.empty(H, P, d, device="cuda")
     refused(lambda: raw(lib.sa_sketch_bwd_tokenwise, t["K"], t["V"], t["cu_seqlens"], B, N, t["Q"], H, P, d,
                         spec.scale, 1, None, None, t["dsketch"], *outs, dQ, ws, ws.numel(), stream()))
+
+
+@pytest.mark.parametrize("per_user_q", [False, True])
+@pytest.mark.parametrize("P,d", SHAPES, ids=lambda x: str(x))
+def test_dq_may_start_anywhere(cuda_lib, P, d, per_user_q):
+    spec, t = inputs(P, d, per_user_q=per_user_q)
+    a = (t["K"], t["V"], t["cu_seqlens"], t["Q"], t["dsketch"], spec.scale)
+    want = binding.sa_sketch_bwd(*a)
+    got = binding.sa_sketch_bwd(*a, outs=(torch.empty_like(t["K"]), torch.empty_like(t["K"]), off(want[2])))
+    assert all(torch.equal(x, y) for x, y in zip(got, want))
+
+
+# users of one tile, which one worker writes whole, and one cut across workers
+LENS = [60] * 300 + [3000]
+
+
+@pytest.mark.parametrize("P,d", [(128, 64), (256, 64), (512, 64), (1024, 64), (128, 128), (512, 128)],
+                         ids=lambda x: str(x))
+def test_sketch_may_start_anywhere(cuda_lib, P, d):
+    spec, t = inputs(P, d, lens=LENS)
+    a = (t["K"], t["V"], t["cu_seqlens"], t["Q"], spec.scale)
+    want = binding.sa_sketch_fwd(*a)
+    assert torch.equal(binding.sa_sketch_fwd(*a, out=off(want)), want)
+
+
+@pytest.mark.parametrize("P,d", [(256, 64), (384, 64), (512, 128)], ids=lambda x: str(x))
+def test_tokenwise_sketch_may_start_anywhere(cuda_lib, P, d):
+    spec, t = inputs(P, d, lens=LENS)
+    lib, N, B, H = binding.load(), t["K"].shape[0], len(LENS), 2
+    want = binding.sa_sketch_fwd_tokenwise(t["K"], t["V"], t["cu_seqlens"], t["Q"], spec.scale)
+    ws = torch.empty(lib.sa_workspace_size_tokenwise(B, N, H, P, d, 1, 0), dtype=torch.uint8, device="cuda")
+    sketch = off(want)
+    raw(lib.sa_sketch_fwd_tokenwise, t["K"], t["V"], t["cu_seqlens"], B, N, t["Q"], H, P, d, spec.scale, 1, sketch,
+        None, ws, ws.numel(), stream())
+    assert torch.equal(sketch, want)
