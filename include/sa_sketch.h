@@ -25,8 +25,8 @@
  *     are float32.  Element offsets are 64-bit.
  *   - K, V and Q (X and Wk of the key projection) start on 16-byte boundaries.
  *     Where the tensor cores serve the call (bf16, d in {64, 128}, P in {128, 256,
- *     512, 1024, 2048}; for the token-wise variant see there) so do dK, dV and dX.
- *     Others are refused with SA_ERR_INVALID_ARG.  The sketch, lse and dQ
+ *     512, 1024, 2048}; for the token-wise variant see there) so do dK, dV, dX and
+ *     dsketch.  Others are refused with SA_ERR_INVALID_ARG.  The sketch, lse and dQ
  *     may start on any 4 bytes.
  *   - K, V   : [N, H, d]   packed rows of all users, N = cu_seqlens[B]
  *     Q      : [H, P, d]   prototypes

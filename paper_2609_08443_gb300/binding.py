@@ -514,7 +514,10 @@ class SketchAttention(torch.autograd.Function):
     @staticmethod
     def backward(ctx, dsketch):
         K, V, cu, Q, lse = ctx.saved_tensors
-        dK, dV, dQ = sa_sketch_bwd(K, V, cu, Q, dsketch.contiguous(), ctx.scale, lse=lse)
+        dsketch = dsketch.contiguous()
+        if dsketch.data_ptr() % 16:  # a view into a larger gradient (of a cat, say)
+            dsketch = dsketch.clone()
+        dK, dV, dQ = sa_sketch_bwd(K, V, cu, Q, dsketch, ctx.scale, lse=lse)
         return dK, dV, None, dQ.to(Q.dtype), None
 
 

@@ -315,8 +315,11 @@ sa_status bwd_check(const void* K, const void* V, const int32_t* cu_seqlens, int
                     const float* dQ, const void* workspace, size_t ws_bytes, int uq, Plan* plan) {
   if (!dsketch || !dQ || (N > 0 && (!dK || !dV))) return SA_ERR_INVALID_ARG;
   SA_TRY(check_common(K, V, cu_seqlens, B, N, Q, H, P, d, scale, dt, workspace, ws_bytes, true, uq, plan));
-  // 16-byte stores and TMA stores
-  if (plan->bwd_path == Path::TcBwd && N > 0 && (!aligned16(dK) || !aligned16(dV))) return SA_ERR_INVALID_ARG;
+  if (plan->bwd_path == Path::TcBwd) {
+    if (N > 0 && (!aligned16(dK) || !aligned16(dV))) return SA_ERR_INVALID_ARG;  // 16-byte stores and TMA stores
+    // 16-byte loads (of the bf16 copy even with no tokens)
+    if ((N > 0 || sa::tc_bwd_split(P, d)) && !aligned16(dsketch)) return SA_ERR_INVALID_ARG;
+  }
   return SA_OK;
 }
 

@@ -73,6 +73,15 @@ def test_tokenwise_gradient_rows(cuda_lib, which):
                         spec.scale, 1, None, None, t["dsketch"], *outs, dQ, ws, ws.numel(), stream()))
 
 
+@pytest.mark.parametrize("P,d", SHAPES, ids=lambda x: str(x))
+def test_dsketch(cuda_lib, P, d):
+    spec, t = inputs(P, d)
+    a = (t["K"], t["V"], t["cu_seqlens"], t["Q"])
+    refused(lambda: binding.sa_sketch_bwd(*a, off(t["dsketch"]), spec.scale))
+    Wk = torch.zeros(2, d, d, dtype=torch.bfloat16, device="cuda")
+    refused(lambda: binding.sa_sketch_bwd_x(t["K"], t["cu_seqlens"], t["Q"], Wk, off(t["dsketch"]), spec.scale))
+
+
 @pytest.mark.parametrize("per_user_q", [False, True])
 @pytest.mark.parametrize("P,d", SHAPES, ids=lambda x: str(x))
 def test_dq_may_start_anywhere(cuda_lib, P, d, per_user_q):
@@ -106,3 +115,17 @@ def test_tokenwise_sketch_may_start_anywhere(cuda_lib, P, d):
     raw(lib.sa_sketch_fwd_tokenwise, t["K"], t["V"], t["cu_seqlens"], B, N, t["Q"], H, P, d, spec.scale, 1, sketch,
         None, ws, ws.numel(), stream())
     assert torch.equal(sketch, want)
+
+
+@pytest.mark.parametrize("P,d", [(256, 64), (512, 128)], ids=lambda x: str(x))
+def test_gradient_of_a_cat(cuda_lib, P, d):
+    """autograd hands a sketch inside a cat a view of the cat's gradient."""
+    spec, t = inputs(P, d)
+    grads = []
+    for pad in (0, 1):
+        leaves = [t[k].clone().requires_grad_(True) for k in ("K", "V", "Q")]
+        s = binding.sa_sketch(leaves[0], leaves[1], t["cu_seqlens"], leaves[2], spec.scale)
+        row = torch.cat([torch.zeros(pad, device="cuda"), s.flatten()])
+        row.backward(torch.cat([torch.zeros(pad, device="cuda"), t["dsketch"].flatten()]))
+        grads.append([x.grad for x in leaves])
+    assert all(torch.equal(x, y) for x, y in zip(*grads))
