@@ -442,6 +442,9 @@ sa_status sa_sketch_fwd_x(const void* X, const int32_t* cu_seqlens, int B, int64
   if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0 || !aligned16(Wk)) return SA_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   void* Qf = static_cast<char*>(workspace) + base;
+  Plan plan;
+  if (!sketch) return SA_ERR_INVALID_ARG;
+  SA_TRY(check_common(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, workspace, base, false, 0, &plan));
   SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_fold_wk(Q, Wk, H, P, d, dt, Qf, st); }));
   return fwd_impl(X, X, cu_seqlens, B, N, Qf, H, P, d, scale, dt, sketch, lse, workspace, base, stream, 0);
 }
