@@ -169,6 +169,8 @@ sa::Args make_args(const void* K, const void* V, const int32_t* cu, int B, int64
   a.dq_partial = reinterpret_cast<float*>(base + L.dq_partial);
   a.lse_scratch = reinterpret_cast<float*>(base + L.lse);
   a.lse_part = reinterpret_cast<float2*>(base + L.lse_part);
+  a.lse_ts = H;
+  a.lse_hs = 1;
   a.uq = 0;
   a.dq_user = nullptr;
   a.sum_dx = 0;
@@ -347,9 +349,14 @@ sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
   char* base = static_cast<char*>(workspace);
   SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_plan(a, plan.T_bwd, st); }));
   if (folded) SA_TRY(fold_negative_scale(a, plan.lay, st));
+  const bool split = plan.bwd_path == Path::TcBwd && sa::tc_bwd_split(P, d);
   const float* l = lse;
   if (!l) {
-    float* scratch = reinterpret_cast<float*>(base + plan.lay.lse);
+    float* scratch = a.lse_scratch;
+    if (split) {  // the first of each float2 [H][N] (lse, D)
+      a.lse_ts = 2;
+      a.lse_hs = 2 * N;
+    }
     if (plan.bwd_path == Path::TcBwd) {
       SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_tc_lse(a, scratch, st); }));
     } else {
@@ -357,15 +364,15 @@ sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
     }
     l = scratch;
   }
-  if (plan.bwd_path == Path::TcBwd && sa::tc_bwd_split(P, d)) {
+  if (split) {
     // token side (dV, dK, D_i) over all prototypes, then dQ per prototype slice
     __nv_bfloat16* gbf = reinterpret_cast<__nv_bfloat16*>(base + plan.lay.gbf);
-    float* Dco = reinterpret_cast<float*>(base + plan.lay.dcoef);
+    float* tokv = a.lse_scratch;  // float2 [H][N] (lse log2 e, D)
     const int Wq = sa::tc_bwd_dq_workers(sa::tcc::device_sm_count(), P);
     SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_tc_g_bf16(a, dsketch, gbf, st); }));
     SA_TRY(launch(SA_KERNEL_BWD_MAIN, st,
-                  [&] { return sa::launch_tc_bwd_tok(a, plan.W_bwd, dsketch, gbf, l, Dco, dK, dV, st); }));
-    SA_TRY(launch(SA_KERNEL_BWD_DQ, st, [&] { return sa::launch_tc_bwd_dq(a, Wq, dsketch, l, Dco, st); }));
+                  [&] { return sa::launch_tc_bwd_tok(a, plan.W_bwd, dsketch, gbf, l, tokv, dK, dV, st); }));
+    SA_TRY(launch(SA_KERNEL_BWD_DQ, st, [&] { return sa::launch_tc_bwd_dq(a, Wq, dsketch, l, tokv, st); }));
     return finalize_dq(Wq);
   }
   if (plan.bwd_path == Path::TcBwd) {

@@ -46,9 +46,11 @@ struct WsLayout {
   size_t partial;      // fp32 [W][2][P][d]: sketch pieces of cut segments
   size_t dq_partial;   // fp32 [W][H][P][d]: per-worker dQ per head (bwd)
   size_t lse;          // fp32 [N][H]: lse scratch when the caller passes none
-  // bwd: D_i = dV_i . v_i, fp32 [N][H] on the CUDA cores; on the tensor cores with
-  // the token's lse beside it, float2 [H][N] (lse log2 e, D_i), so that a tile's
-  // tokens are one contiguous copy for the dQ kernel
+  // bwd on the CUDA cores: D_i = dV_i . v_i, fp32 [N][H].  Where prototype slices compute
+  // dQ on the tensor cores this section and `lse` are one: float2 [H][N] (lse log2 e, D_i)
+  // from `lse` on, so that a tile's tokens are one contiguous copy for the dQ kernel.
+  // Without the caller's lse the first of each pair holds the token's lse until the token
+  // side, which reads it, writes the pair.
   size_t dcoef;
   size_t gbf;          // bf16 [B][H][P][d]: dsketch copy streamed by TMA (split backward)
   size_t lse_part;     // float2 [N][H][P / 512]: per-slice (max, sum) of the lse pass (P >= 1024)
@@ -68,7 +70,7 @@ SA_HD WsLayout ws_layout(int B, int64_t N, int H, int P, int d, int W, bool bwd)
   L.lse = off;
   off = align256(off + sizeof(float) * size_t(N) * size_t(H));
   L.dcoef = off;
-  if (bwd) off = align256(off + 2 * sizeof(float) * size_t(N) * size_t(H));
+  if (bwd) off = align256(off + sizeof(float) * size_t(N) * size_t(H));
   L.gbf = off;
   if (bwd && ((d == 128 && P > 128) || (d == 64 && P > 256)))
     off = align256(off + 2 * size_t(B) * size_t(H) * size_t(P) * size_t(d));

@@ -19,7 +19,8 @@ struct Args {
   int64_t* prefix;     // per-head tile prefix [B + 1]
   float* partial;      // [W][2][P][d]
   float* dq_partial;   // [W][H][P][d]
-  float* lse_scratch;  // [N][H] workspace copy of lse when the caller passes none
+  float* lse_scratch;  // workspace section of the lse when the caller passes none
+  int64_t lse_ts, lse_hs;  // the call's lse of token t, head h lies at [t lse_ts + h lse_hs]
   float2* lse_part;    // [N][H][slices] per-slice (max, sum) of the lse pass when P >= 1024
   int uq;              // 1: per-user queries Q[B][H][P][d] and dQ[B][H][P][d] (stacked refinement)
   float* dq_user;      // per-user queries: the caller's dQ[B][H][P][d] (whole segments go there)

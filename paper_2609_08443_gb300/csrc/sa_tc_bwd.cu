@@ -116,7 +116,7 @@ __host__ __device__ constexpr int tok_da_col() {
 __device__ __forceinline__ int tok_kv_pair(int) { return 0; }
 __device__ __forceinline__ int tok_qg_pair(int, int c) { return 1 + (c & 1); }
 
-// TW = false: prototype-wise weights (Sec. 3.1), lse per token [N][H]; Dco is
+// TW = false: prototype-wise weights (Sec. 3.1), lse per token and head; Dco is
 // written here, float2 [H][N] (lse log2 e, D_i).  TW = true: token-wise weights (Sec. 5.1), lse and Dco
 // per prototype [B][H][P] (both read), so dS = A o (dA - D_j) goes to shared
 // memory in place of E and dK = scale dS Q needs no qbar.
@@ -124,8 +124,8 @@ __device__ __forceinline__ int tok_qg_pair(int, int c) { return 1 + (c & 1); }
 template <int D, int P, bool TW, bool SUM>
 __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmQ,
                                              const CUtensorMap& tmG, const CUtensorMap& tmDK,
-                                             const CUtensorMap& tmDV, const Args& a, const float* __restrict__ lse,
-                                             float* __restrict__ Dco, __nv_bfloat16* __restrict__ dK,
+                                             const CUtensorMap& tmDV, const Args& a, const float* lse,
+                                             float* Dco, __nv_bfloat16* __restrict__ dK,
                                              __nv_bfloat16* __restrict__ dV) {
   using C = TokCfg<D, P>;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -390,7 +390,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
         ++epi;
         return r;
       };
-      float lse_cur = (!TW && row < cur.n) ? lse[(cur.tok0 + row) * a.H + cur.h] : 0.f;
+      float lse_cur = (!TW && row < cur.n) ? load_token_lse(lse, a, cur.tok0 + row, cur.h) : 0.f;
       for (int li = 0; li < ntiles && ok; ++li) {
         const bool valid = row < cur.n;
         const int64_t tok = cur.tok0 + row;
@@ -399,7 +399,7 @@ __device__ __forceinline__ void bwd_tok_body(const CUtensorMap& tmK, const CUten
           int64_t t0n;
           int nn, hn;
           cur.peek_next(t0n, nn, hn);
-          lse_cur = row < nn ? lse[(t0n + row) * a.H + hn] : 0.f;
+          lse_cur = row < nn ? load_token_lse(lse, a, t0n + row, hn) : 0.f;
         }
         // token-wise: this segment's per-prototype lse and D_j (the same for
         // every thread: broadcast loads)
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_bwd_tok_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
                       const __grid_constant__ CUtensorMap tmDK, const __grid_constant__ CUtensorMap tmDV, Args a,
-                      const float* __restrict__ lse, float* __restrict__ Dco, __nv_bfloat16* __restrict__ dK,
+                      const float* lse, float* Dco, __nv_bfloat16* __restrict__ dK,
                       __nv_bfloat16* __restrict__ dV) {
   bwd_tok_body<D, P, false, SUM>(tmK, tmV, tmQ, tmG, tmDK, tmDV, a, lse, Dco, dK, dV);
 }

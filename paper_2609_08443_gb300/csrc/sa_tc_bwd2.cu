@@ -143,7 +143,7 @@ template <int D, int P, bool FUSE, bool SUM>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_bwd2_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                    const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
-                   Args a, const float* __restrict__ dsk, const float* __restrict__ lse, float* __restrict__ Dco,
+                   Args a, const float* __restrict__ dsk, const float* lse, float* Dco,
                    __nv_bfloat16* __restrict__ dK, __nv_bfloat16* __restrict__ dV) {
   using C = SCfg<D, P, FUSE, SUM>;
   constexpr int NCH = C::NCH, ND = C::ND, BLK = C::BLK;
@@ -690,7 +690,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // which chunk of sweep 1 the last tile's outputs follow: the first where dV needs
     // their accumulator, else the second, whose wait covers theirs
     constexpr int kFin = C::SHARED_ACC || NCH == 1 ? 0 : 1;
-    auto load_lse = [&](const Tile& o) { return row < o.n ? lse[(o.tok0 + row) * a.H + o.h] : INFINITY; };
+    auto load_lse = [&](const Tile& o) {
+      if (row >= o.n) return float(INFINITY);
+      return FUSE ? __ldg(lse + (o.tok0 + row) * a.H + o.h) : load_token_lse(lse, a, o.tok0 + row, o.h);
+    };
     ok = wwait(i_full, 0, 0xF12);
     Tile cur{}, prev{};
     if (ok) cur = read_tile(0);

@@ -127,6 +127,14 @@ __device__ __forceinline__ bool cta_leaves(void* ws, uint32_t smem_base, uint32_
   return __syncthreads_or(misaligned || ws_failed(ws)) != 0;
 }
 
+// The lse of one (token, head).  Volatile: it may lie where the token side writes the pair
+// (lse log2 e, D) of the same token later, so it is read exactly once, before.
+__device__ __forceinline__ float load_token_lse(const float* lse, const Args& a, int64_t tok, int h) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(lse + tok * a.lse_ts + h * a.lse_hs));
+  return x;
+}
+
 // Where a worker's dQ block of prototypes [p0, p0 + PS) for the tiles ending
 // at walker position w goes.  Shared queries: the worker's partial of head h
 // ([W][H][P][d], summed over workers afterwards).  Per-user queries: dQ[b, h]

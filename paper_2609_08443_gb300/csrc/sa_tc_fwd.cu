@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float Z = z * ex2((m - M) * c2) + o.y * ex2((o.x - M) * c2);
           const int64_t th = (cur.tok0 + row) * a.H + cur.h;
           if (NS == 1)
-            lse_out[th] = M * a.scale + logf(Z);
+            lse_out[(cur.tok0 + row) * a.lse_ts + cur.h * a.lse_hs] = M * a.scale + logf(Z);
           else
             part_out[th * NS + slice] = make_float2(M, Z);
         }
@@ -777,9 +777,10 @@ static cudaError_t launch_lse_t(const Args& a, int W, float* lse_out, float2* pa
   return cudaGetLastError();
 }
 
-// lse[t, h] from the NS per-slice partials (max, sum), folded in slice order.
-__global__ void combine_lse_kernel(const float2* __restrict__ part, int NS, int64_t nth, float scale,
-                                   float* __restrict__ lse, const void* ws) {
+// lse of (token, head) i = t H + h from the NS per-slice partials (max, sum), folded in
+// slice order.
+__global__ void combine_lse_kernel(const float2* __restrict__ part, int NS, int64_t nth, int H, float scale,
+                                   float* __restrict__ lse, int64_t ts, int64_t hs, const void* ws) {
   if (ws_failed(ws)) return;
   const float c2 = scale * 1.4426950408889634f;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < nth; i += int64_t(gridDim.x) * blockDim.x) {
@@ -789,7 +790,7 @@ __global__ void combine_lse_kernel(const float2* __restrict__ part, int NS, int6
       const float M = fmaxf(acc.x, y.x);
       acc = make_float2(M, acc.y * ex2((acc.x - M) * c2) + y.y * ex2((y.x - M) * c2));
     }
-    lse[i] = acc.x * scale + logf(acc.y);
+    lse[hs == 1 ? i : (i / H) * ts + (i % H) * hs] = acc.x * scale + logf(acc.y);
   }
 }
 
@@ -852,7 +853,8 @@ cudaError_t launch_tc_lse(const Args& a, float* lse, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const int NS = a.P / tc_lse_slice(a.P, a.d);
   if (NS > 1) {
-    tcf::combine_lse_kernel<<<1024, 256, 0, st>>>(a.lse_part, NS, a.N * a.H, a.scale, lse, a.ws);
+    tcf::combine_lse_kernel<<<1024, 256, 0, st>>>(a.lse_part, NS, a.N * a.H, a.H, a.scale, lse, a.lse_ts, a.lse_hs,
+                                                  a.ws);
     e = cudaGetLastError();
   }
   return e;
