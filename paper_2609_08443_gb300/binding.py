@@ -7,9 +7,11 @@ built or cannot be loaded, every call raises: there is no CPU fallback.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import math
 import os
+import threading
 from typing import Optional, Tuple
 
 import torch
@@ -111,7 +113,7 @@ def _dt(t: torch.Tensor) -> int:
 
 
 # The argument types are declared, so addresses pass as plain integers; together with
-# the raw stream handle and a workspace looked up by the tensor's device this takes a
+# the raw stream handle and a workspace looked up by device and stream this takes a
 # forward call of one small user from 34 to 23 us of host time (9 us of it the
 # library's launches), which is what paces such calls.
 def _ptr(t: Optional[torch.Tensor]):
@@ -185,19 +187,52 @@ def sa_get_device_error(workspace: torch.Tensor) -> int:
     return int(load().sa_get_device_error(_ptr(workspace), _stream(workspace.device)))
 
 
-_ws_cache = {}
+# One workspace per device and stream: the calls that share one are ordered by their
+# stream, and so is whatever gets its memory once it is replaced (torch gives a freed block
+# back to the stream that it was allocated on).  Two threads on one stream take turns: a
+# call holds the lock until all of its kernels are enqueued.  Beyond _WS_MAX the oldest goes.
+_WS_MAX = 16
+_ws_cache = {}  # (device index, raw stream) -> [lock, buffer]
+_ws_mutex = threading.Lock()
+_NO_LOCK = contextlib.nullcontext()
+
+
+def _ws_entry(key):
+    with _ws_mutex:
+        entry = _ws_cache.get(key)
+        if entry is None:
+            while len(_ws_cache) >= _WS_MAX:
+                del _ws_cache[next(iter(_ws_cache))]
+            entry = _ws_cache[key] = [threading.RLock(), None]
+    return entry
+
+
+def _workspace(nbytes: int, device: torch.device, ws: Optional[torch.Tensor] = None):
+    """(workspace, raw stream, lock to hold while the call is enqueued): the caller's ``ws``,
+    else the one of ``device``'s current stream; under stream capture a new one, so that it
+    belongs to the graph and lives as long."""
+    index = device.index
+    if index is None:
+        index = torch.cuda.current_device()
+    stream = torch._C._cuda_getCurrentRawStream(index)
+    if ws is not None:
+        return ws, stream, _NO_LOCK
+    if torch.cuda.is_current_stream_capturing():
+        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device), stream, _NO_LOCK
+    entry = _ws_cache.get((index, stream))
+    if entry is None:
+        entry = _ws_entry((index, stream))
+    buf = entry[1]
+    if buf is None or buf.numel() < nbytes:
+        buf = entry[1] = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    return buf, stream, entry[0]
 
 
 def workspace(nbytes: int, device) -> torch.Tensor:
-    """A cached uint8 device buffer of at least ``nbytes`` (allocated by torch)."""
-    dev = torch.device(device)
-    if dev.index is None:
-        dev = torch.device(dev.type, torch.cuda.current_device())
-    buf = _ws_cache.get(dev)
-    if buf is None or buf.numel() < nbytes:
-        buf = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=dev)
-        _ws_cache[dev] = buf
-    return buf
+    """The cached uint8 buffer of ``device``'s current stream, of at least ``nbytes``
+    (allocated by torch)."""
+    torch.cuda.init()
+    return _workspace(nbytes, torch.device(device))[0]
 
 
 def sa_sketch_fwd(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.Tensor, Q: torch.Tensor,
@@ -220,9 +255,10 @@ def sa_sketch_fwd(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.Tensor, Q:
     need = lib.sa_workspace_size(B, N, H, P, d, dt, 0)
     if need == 0:
         raise SketchError(2, "sa_workspace_size")
-    w = ws if ws is not None else workspace(need, K.device)
-    st = entry(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
-               _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), _stream(K.device))
+    w, stream, lock = _workspace(need, K.device, ws)
+    with lock:
+        st = entry(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
+                   _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_fwd_per_user" if Q.dim() == 4 else "sa_sketch_fwd")
     return (sketch, lse) if want_lse or lse_out is not None else sketch
 
@@ -252,9 +288,10 @@ def sa_sketch_bwd(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.Tensor, Q:
     need = lib.sa_workspace_size(B, N, H, P, d, dt, 1)
     if need == 0:
         raise SketchError(2, "sa_workspace_size")
-    w = ws if ws is not None else workspace(need, K.device)
-    st = entry(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
-               _ptr(dsketch), _ptr(lse), _ptr(dK), _ptr(dV), _ptr(dQ), _ptr(w), w.numel(), _stream(K.device))
+    w, stream, lock = _workspace(need, K.device, ws)
+    with lock:
+        st = entry(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
+                   _ptr(dsketch), _ptr(lse), _ptr(dK), _ptr(dV), _ptr(dQ), _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_bwd_per_user" if Q.dim() == 4 else "sa_sketch_bwd")
     return dK, dV, dQ
 
@@ -340,9 +377,10 @@ def sa_sketch_fwd_x(X: torch.Tensor, cu_seqlens: torch.Tensor, Q: torch.Tensor, 
     need = lib.sa_workspace_size_x(B, N, H, P, d, dt, 0)
     if need == 0:
         raise SketchError(2, "sa_workspace_size_x")
-    w = ws if ws is not None else workspace(need, X.device)
-    st = lib.sa_sketch_fwd_x(_ptr(X), _ptr(cu_seqlens), B, N, _ptr(Q), _ptr(Wk), H, P, d, scale, dt,
-                             _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), _stream(X.device))
+    w, stream, lock = _workspace(need, X.device, ws)
+    with lock:
+        st = lib.sa_sketch_fwd_x(_ptr(X), _ptr(cu_seqlens), B, N, _ptr(Q), _ptr(Wk), H, P, d, scale, dt,
+                                 _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_fwd_x")
     return (sketch, lse) if want_lse else sketch
 
@@ -366,10 +404,11 @@ def sa_sketch_bwd_x(X: torch.Tensor, cu_seqlens: torch.Tensor, Q: torch.Tensor, 
     need = lib.sa_workspace_size_x(B, N, H, P, d, dt, 1)
     if need == 0:
         raise SketchError(2, "sa_workspace_size_x")
-    w = ws if ws is not None else workspace(need, X.device)
-    st = lib.sa_sketch_bwd_x(_ptr(X), _ptr(cu_seqlens), B, N, _ptr(Q), _ptr(Wk), H, P, d, scale, dt,
-                             _ptr(dsketch), _ptr(lse), _ptr(dX), _ptr(dQ), _ptr(dWk), _ptr(w), w.numel(),
-                             _stream(X.device))
+    w, stream, lock = _workspace(need, X.device, ws)
+    with lock:
+        st = lib.sa_sketch_bwd_x(_ptr(X), _ptr(cu_seqlens), B, N, _ptr(Q), _ptr(Wk), H, P, d, scale, dt,
+                                 _ptr(dsketch), _ptr(lse), _ptr(dX), _ptr(dQ), _ptr(dWk), _ptr(w), w.numel(),
+                                 stream)
     _check(st, "sa_sketch_bwd_x")
     return dX, dQ, dWk
 
@@ -393,9 +432,10 @@ def sa_sketch_fwd_tokenwise(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.
     need = lib.sa_workspace_size_tokenwise(B, N, H, P, d, dt, 0)
     if need == 0:
         raise SketchError(2, "sa_workspace_size_tokenwise")
-    w = ws if ws is not None else workspace(need, K.device)
-    st = lib.sa_sketch_fwd_tokenwise(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
-                                     _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), _stream(K.device))
+    w, stream, lock = _workspace(need, K.device, ws)
+    with lock:
+        st = lib.sa_sketch_fwd_tokenwise(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
+                                         _ptr(sketch), _ptr(lse), _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_fwd_tokenwise")
     return (sketch, lse) if want_lse else sketch
 
@@ -424,10 +464,11 @@ def sa_sketch_bwd_tokenwise(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.
     need = lib.sa_workspace_size_tokenwise(B, N, H, P, d, dt, 1)
     if need == 0:
         raise SketchError(2, "sa_workspace_size_tokenwise")
-    w = ws if ws is not None else workspace(need, K.device)
-    st = lib.sa_sketch_bwd_tokenwise(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
-                                     _ptr(sketch), _ptr(lse), _ptr(dsketch), _ptr(dK), _ptr(dV), _ptr(dQ),
-                                     _ptr(w), w.numel(), _stream(K.device))
+    w, stream, lock = _workspace(need, K.device, ws)
+    with lock:
+        st = lib.sa_sketch_bwd_tokenwise(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
+                                         _ptr(sketch), _ptr(lse), _ptr(dsketch), _ptr(dK), _ptr(dV), _ptr(dQ),
+                                         _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_bwd_tokenwise")
     return dK, dV, dQ
 
@@ -459,13 +500,15 @@ def sa_sketch_step_host(K: torch.Tensor, V: torch.Tensor, cu_seqlens: torch.Tens
                 torch.empty_like(K, pin_memory=pin), torch.empty_like(V, pin_memory=pin),
                 torch.empty((H, P, d), dtype=torch.float32, pin_memory=pin))
     sketch, dK, dV, dQ = outs
+    torch.cuda.init()
     need = lib.sa_step_host_workspace_size(_ptr(cu_seqlens), B, H, P, d, dt, int(chunk_tokens))
     if need == 0:
         raise SketchError(2, "sa_step_host_workspace_size")
-    w = ws if ws is not None else workspace(need, dev)
-    st = lib.sa_sketch_step_host(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
-                                 _ptr(dsketch), _ptr(sketch), _ptr(dK), _ptr(dV), _ptr(dQ), int(chunk_tokens),
-                                 _ptr(w), w.numel(), _stream(dev))
+    w, stream, lock = _workspace(need, dev, ws)
+    with lock:
+        st = lib.sa_sketch_step_host(_ptr(K), _ptr(V), _ptr(cu_seqlens), B, N, _ptr(Q), H, P, d, scale, dt,
+                                     _ptr(dsketch), _ptr(sketch), _ptr(dK), _ptr(dV), _ptr(dQ), int(chunk_tokens),
+                                     _ptr(w), w.numel(), stream)
     _check(st, "sa_sketch_step_host")
     torch.cuda.current_stream(dev).synchronize()
     return sketch, dK, dV, dQ
