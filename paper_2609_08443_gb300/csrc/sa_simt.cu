@@ -197,10 +197,13 @@ __device__ __forceinline__ int col_of(int cg, int m) {
 }
 
 // Row statistics of the scores seen so far, per token of this thread (its share of
-// the prototypes): maximum and sum of exp(s - max).
+// the prototypes): maximum m and sum of exp(s - shift(m)).  An infinite maximum is no
+// shift: of -inf alone the sum is 0, and an overflowed score makes it, and the lse, +inf,
+// so that the other prototypes' weights are exact zeros; a NaN reaches the sum either way.
 struct RowStat {
   float m[kTok], z[kTok];
 };
+__device__ __forceinline__ float shift(float m) { return fabsf(m) == INFINITY ? 0.f : m; }
 
 // (max, sum) of every token over all threads that share it, to red[2][32]
 __device__ __forceinline__ void reduce_stat(RowStat& r, float (*red)[2][32]) {
@@ -211,8 +214,8 @@ __device__ __forceinline__ void reduce_stat(RowStat& r, float (*red)[2][32]) {
     for (int o = 8; o < 32; o <<= 1) {
       const float m2 = __shfl_xor_sync(0xffffffffu, r.m[i], o), z2 = __shfl_xor_sync(0xffffffffu, r.z[i], o);
       const float mm = fmaxf(r.m[i], m2);
-      const float za = r.z[i] == 0.f ? 0.f : r.z[i] * expf(r.m[i] - mm);
-      const float zb = z2 == 0.f ? 0.f : z2 * expf(m2 - mm);
+      const float za = r.z[i] == 0.f ? 0.f : r.z[i] * expf(r.m[i] - shift(mm));
+      const float zb = z2 == 0.f ? 0.f : z2 * expf(m2 - shift(mm));
       r.m[i] = mm;
       r.z[i] = za + zb;
     }
@@ -262,7 +265,7 @@ __global__ void __launch_bounds__(SNT) simt_lse_kernel(Args a, float* __restrict
         s[i][j] = pro_of(j) < np ? s[i][j] * a.scale : -INFINITY;
         m = fmaxf(m, s[i][j]);
       }
-      const float sh = m == -INFINITY ? 0.f : m;  // no finite score yet: a NaN still reaches the sum
+      const float sh = shift(m);
       float z = rs.z[i] * expf(rs.m[i] - sh);
 #pragma unroll
       for (int j = 0; j < kPro; ++j) z += expf(s[i][j] - sh);
@@ -280,7 +283,7 @@ __global__ void __launch_bounds__(SNT) simt_lse_kernel(Args a, float* __restrict
     float z = 0.f;
 #pragma unroll
     for (int w = 0; w < SNT / 32; ++w)
-      if (red[w][1][tid] != 0.f) z += red[w][1][tid] * expf(red[w][0][tid] - m);
+      if (red[w][1][tid] != 0.f) z += red[w][1][tid] * expf(red[w][0][tid] - shift(m));
     lse[(r.tok0 + tid) * H + r.h] = m + logf(z);
   }
 }
