@@ -103,8 +103,9 @@ struct Acc {
 };
 
 // Users without tokens get zero rows (token-wise: lse = -inf).  Each is cut into slices, a
-// head's worth or less, so that a few users with much to clear still take the whole chip;
-// the threads of a block look at its next 256 (user, slice) items at once.  A forward
+// head's worth or less but a store of every thread at least, so that a few users with much
+// to clear still take the whole chip; the threads of a block look at its next 256 (user,
+// slice) items at once.  A forward
 // call of one such user with 64 heads, P = 2048, d = 128 (67 MB): 1022 us when one block
 // cleared it, 18.9 us this way.
 template <int V, int KIND>
@@ -112,7 +113,7 @@ __device__ __forceinline__ void zero_empty_users(const FinArgs& a) {
   __shared__ uint32_t empty_s[kFinWarps];
   const int tid = threadIdx.x, grid = int(gridDim.x);
   const int64_t len = int64_t(a.H) * a.P * a.d;
-  const int slices = max(a.H, (grid + a.B - 1) / a.B);
+  const int slices = int(min(int64_t(max(a.H, (grid + a.B - 1) / a.B)), max(int64_t(1), len / (kFinThreads * V))));
   const int64_t per = ((len + slices - 1) / slices + 3) & ~int64_t(3), items = int64_t(a.B) * slices;
   for (int64_t base = blockIdx.x; base < items; base += int64_t(grid) * kFinThreads) {
     const int64_t mine = base + int64_t(tid) * grid;

@@ -604,8 +604,12 @@ static cudaError_t run(Fn* fn, dim3 grid, size_t floats, cudaStream_t st, Xs... 
   return cudaGetLastError();
 }
 
-// one block per tile: H x ceil(L_b / 32) summed over the users is at most this
-static unsigned max_tiles(const Args& a) { return unsigned(int64_t(a.H) * ((a.N + ST - 1) / ST + a.B)); }
+// one block per tile: H x ceil(L_b / 32) summed over the users, of whom at most N have
+// tokens, is at most this
+static unsigned max_tiles(const Args& a) {
+  const int64_t users = a.N < a.B ? a.N : a.B;
+  return unsigned(int64_t(a.H) * ((a.N + (ST - 1) * users) / ST));
+}
 
 cudaError_t launch_simt_lse(const Args& a, float* lse, cudaStream_t st) {
   if (a.N == 0) return cudaSuccess;
