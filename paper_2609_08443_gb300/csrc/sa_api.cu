@@ -371,7 +371,7 @@ sa_status bwd_impl(const void* K, const void* V, const int32_t* cu_seqlens, int 
     const int Wq = sa::tc_bwd_dq_workers(sa::tcc::device_sm_count(), P);
     SA_TRY(launch(SA_KERNEL_AUX, st, [&] { return sa::launch_tc_g_bf16(a, dsketch, gbf, st); }));
     SA_TRY(launch(SA_KERNEL_BWD_MAIN, st,
-                  [&] { return sa::launch_tc_bwd_tok(a, plan.W_bwd, dsketch, gbf, l, tokv, dK, dV, st); }));
+                  [&] { return sa::launch_tc_bwd_tok(a, plan.W_bwd, gbf, l, tokv, dK, dV, st); }));
     SA_TRY(launch(SA_KERNEL_BWD_DQ, st, [&] { return sa::launch_tc_bwd_dq(a, Wq, dsketch, l, tokv, st); }));
     return finalize_dq(Wq);
   }

@@ -85,16 +85,6 @@ SA_HD WsLayout ws_layout(int B, int64_t N, int H, int P, int d, int W, bool bwd)
 // ------------------------------------------------------------------ tiling
 SA_HD int64_t range_begin(int64_t total, int W, int w) { return (total * int64_t(w)) / W; }
 
-// Largest worker w with range_begin(w) <= t (so a worker with an empty range
-// never owns a tile).  0 <= t < total.
-SA_HD int owner_of(int64_t total, int W, int64_t t) {
-  int64_t g = (t * int64_t(W)) / (total > 0 ? total : 1);
-  if (g >= W) g = W - 1;
-  while (g + 1 < W && range_begin(total, W, int(g + 1)) <= t) ++g;
-  while (g > 0 && range_begin(total, W, int(g)) > t) --g;
-  return int(g);
-}
-
 // Largest b in [0, B) with prefix[b] <= r (prefix non-decreasing, prefix[0]=0,
 // r < prefix[B]); skips users with no tiles.
 SA_HD int find_user(const int64_t* prefix, int B, int64_t r) {

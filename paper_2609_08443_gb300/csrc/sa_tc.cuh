@@ -20,10 +20,11 @@ int tc_fwd_workers(int num_sms, int P, int d);
 int tc_bwd_workers(int num_sms, int P, int d);
 cudaError_t launch_tc_fwd(const Args& a, int W, float* sketch, float* lse, cudaStream_t st);
 cudaError_t launch_tc_lse(const Args& a, float* lse, cudaStream_t st);
-// d = 128 with P in {256, 512}: token side (dV, dK, D_i) then prototype slices (dQ)
+// token side (dV, dK, D_i), then prototype slices (dQ): d = 128 from P = 256 on, d = 64
+// from P = 512 on
 bool tc_bwd_split(int P, int d);
-cudaError_t launch_tc_bwd_tok(const Args& a, int W, const float* dsk, __nv_bfloat16* gbf, const float* lse,
-                              float* Dco, void* dK, void* dV, cudaStream_t st);
+cudaError_t launch_tc_bwd_tok(const Args& a, int W, const __nv_bfloat16* gbf, const float* lse, float* Dco, void* dK,
+                              void* dV, cudaStream_t st);
 cudaError_t launch_tc_bwd_dq(const Args& a, int W, const float* dsk, const float* lse, const float* Dco,
                              cudaStream_t st);
 int tc_bwd_dq_workers(int num_sms, int P);

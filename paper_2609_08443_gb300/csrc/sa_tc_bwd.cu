@@ -665,9 +665,8 @@ cudaError_t launch_tc_g_bf16(const Args& a, const float* dsk, __nv_bfloat16* gbf
   return cudaGetLastError();
 }
 
-cudaError_t launch_tc_bwd_tok(const Args& a, int W, const float* dsk, __nv_bfloat16* gbf, const float* lse,
-                              float* Dco, void* dK, void* dV, cudaStream_t st) {
-  (void)dsk;
+cudaError_t launch_tc_bwd_tok(const Args& a, int W, const __nv_bfloat16* gbf, const float* lse, float* Dco, void* dK,
+                              void* dV, cudaStream_t st) {
   if (a.N == 0) return cudaSuccess;
   if (a.P <= 512) return launch_tc_bwd2_tok(a, W, gbf, lse, Dco, dK, dV, st);
   if (a.d == 64)

@@ -527,7 +527,10 @@ static cudaError_t launch_dq_t(const Args& a, int W, const float* dsk, const flo
   using C = DCfg<D>;
   CUtensorMap tk, tv;
   if (!make_kv_map(&tk, a.K, a.N, a.H, D) || !make_kv_map(&tv, a.V, a.N, a.H, D)) return cudaErrorInvalidValue;
-  auto fn = TW ? &tc_tw_bwd_dq_kernel<D, C::PS> : &tc_bwd_dq_kernel<D, C::PS>;
+  auto fn = [] {
+    if constexpr (TW) return &tc_tw_bwd_dq_kernel<D, C::PS>;
+    else return &tc_bwd_dq_kernel<D, C::PS>;
+  }();
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   const dim3 grid(W, a.P / C::PS);
