@@ -131,8 +131,8 @@ sa_status sa_sketch_bwd_per_user(const void* K, const void* V, const int32_t* cu
  *     Q  : [H, P, d]  (type `dt`, the projected prototypes P W_Q)
  * Computed as the step with K = V = X and prototypes Q' = Q Wk^T (equal scores:
  * q_j . (x_i Wk) = (q_j Wk^T) . x_i); no K is formed.  The workspace must hold
- * sa_workspace_size_x() bytes (the step's own plus Q', and for the backward dK'
- * and dQ').  Other arguments, results and errors as in sa_sketch_fwd. */
+ * sa_workspace_size_x() bytes (the step's own plus Q', and for the backward dQ'
+ * and, where the CUDA cores serve it, dK').  Other arguments, results and errors as in sa_sketch_fwd. */
 size_t sa_workspace_size_x(int B, int64_t N, int H, int P, int d, sa_dtype dt, int bwd);
 sa_status sa_sketch_fwd_x(const void* X, const int32_t* cu_seqlens, int B, int64_t N, const void* Q,
                           const void* Wk, int H, int P, int d, float scale, sa_dtype dt, float* sketch,

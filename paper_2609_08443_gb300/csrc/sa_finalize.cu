@@ -12,10 +12,11 @@
 // list), and the list's (segment, column range) items are dealt to all blocks.  Segments of up to
 // kFewPieces pieces (a long batch) give each thread one column and its pieces
 // in order; longer chains (a short batch) are split over the block's eight
-// warps, whose sums are added in warp order.  Token-wise segments have [P][d] columns
-// enough for the chip at any length, and their lse and sketch feed the backward's
-// differences, where another order of the sums shows as flipped bf16 roundings: they
-// are always added in piece order, relative to the largest shift.  All orders depend
+// warps, whose sums are added in warp order.  Token-wise lse and sketches feed the backward's
+// differences, where another order of the sums shows as flipped bf16 roundings: their
+// pieces are always added in order, relative to the largest shift, one thread per column
+// (a narrow shape, P = 1 and d = 8 say, leaves the whole chain to two threads, as the
+// kernel before this did).  All orders depend
 // only on the plan, so the result stays bitwise reproducible.  Measured, the
 // calls with the old and with this kernel and nothing else changed: one user of 1531
 // tokens 69.6 and 32.0 us, one fp32 user of 4096 tokens 226 and 65.6 us, the token-wise
@@ -30,6 +31,11 @@ namespace {
 
 constexpr int kFinThreads = 256;
 constexpr int kFinWarps = kFinThreads / 32;
+// Up to four pieces in order, more split.  Forwards at d = 64, P = 256 (at d = 128,
+// P = 512), us, in order and split: two or three pieces a segment 68.5 and 81.6 (92 and
+// 119), five 49.7 and 55.7 (89 and 102), ten 48.4 and 51.1, nineteen 33.4 and 33.4.  The
+// split pays for chains of a hundred (one fp32 user: 226 and 65.6 us with the whole
+// kernel).  The line could lie at 16; it is left at 4, where every sum keeps its order.
 constexpr int kFewPieces = 4;
 
 enum Kind { kSketch = 0, kHeadDq = 1, kTokenwise = 2 };

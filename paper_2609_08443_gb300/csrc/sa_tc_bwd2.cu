@@ -35,9 +35,9 @@
 // chain.  The issuers' chunk loops stay rolled (unrolled, the kernel is 160 KB of code
 // for 99, and slower).  Every wait is bounded (sa_ptx.cuh).
 // Measured, kernel alone: 64 users (1.5M tokens, H = 8, P = 256, d = 64) 3.19 ms with
-// the one-sweep kernel that kept A and dS in shared memory, 2.15 ms now; 16 users of
-// 100K tokens at P = 512, d = 128 6.82 and 6.26 ms; 12 users of 137K tokens with their
-// own queries 0.61 and 0.54 ms.
+// the one-sweep kernel that kept A and dS in shared memory, 2.14 ms now; 16 users of
+// 100K tokens at P = 512, d = 128 6.82 and 6.15 ms; 12 users of 137K tokens with their
+// own queries 0.61 and 0.56 ms.
 #include <cuda.h>
 
 #include "sa_handoff.cuh"

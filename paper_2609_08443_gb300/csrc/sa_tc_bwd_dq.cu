@@ -24,9 +24,10 @@
 // The issuers wait for all that a tile needs in one round of polls and read the next
 // tile's flags a tile ahead: seven waits in turn, 250-450 cycles each although
 // satisfied, had cost 2100 cycles per tile.
-// Measured: 16 users of 100K tokens (H = 8, P = 512, d = 128) 4.37 ms before, 3.79 ms
+// Measured: 16 users of 100K tokens (H = 8, P = 512, d = 128) 4.37 ms before, 3.58 ms
 // now; 12 users, 215K tokens, token-wise 678 and 452 us; P = 1024, 141K tokens, 797
-// and 634 us.
+// and 622 us.  With lse and D as two arrays of their own, copied one by one, the first
+// took 3.92 ms; with lse in natural units, scaled when it is laid out, 3.72.
 // TMEM: per half S 64 (dS over its first 32) and dA 64, G D/2, Q D/2, dQ D columns.
 //
 // Warp roles: 0 tile sequence, loads; 1 issues S and dA, 2 (also TMEM) issues dQ; 3

@@ -18,7 +18,7 @@
 // microseconds of FMA; one thread per output reading its operands from global
 // memory took 265 us (Q') and 171 us (dQ and dW_K together).
 // The step of 12 users (256K tokens, P = 512, d = 128): 3.76 ms with those and
-// the separate dX pass (538 us), 2.40 ms now.
+// the separate dX pass (538 us), 2.40 ms without (2.09 ms with the present backward).
 #include "sa_kernels.cuh"
 
 namespace sa {
